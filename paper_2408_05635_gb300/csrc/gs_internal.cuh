@@ -188,22 +188,18 @@ struct GaussPtrs {
     const void *quats, *log_scales, *logits, *rgb;
 };
 
-// Block-wide sum of two per-thread counters, added once per block to the header.
-__device__ __forceinline__ void count_pairs(uint32_t evals, uint32_t contrib, unsigned long long *e_out,
-                                            unsigned long long *c_out) {
-    __shared__ unsigned long long s_e, s_c;
-    if (threadIdx.x == 0) s_e = s_c = 0ull;
-    __syncthreads();
+// Pair counters of a tile block: every warp adds its lanes' counts to the block's shared
+// totals (zeroed before the block's first barrier), and one thread adds those to the header
+// after the block's last barrier.
+__device__ __forceinline__ void count_warp(uint32_t evals, uint32_t contrib, unsigned long long *s_count) {
     const uint32_t we = __reduce_add_sync(0xffffffffu, evals), wc = __reduce_add_sync(0xffffffffu, contrib);
     if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&s_e, (unsigned long long)we);
-        atomicAdd(&s_c, (unsigned long long)wc);
+        atomicAdd(s_count, (unsigned long long)we);
+        atomicAdd(s_count + 1, (unsigned long long)wc);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(e_out), "l"(s_e) : "memory");
-        asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(c_out), "l"(s_c) : "memory");
-    }
+}
+__device__ __forceinline__ void red_add64(unsigned long long *p, unsigned long long v) {
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 // Fire-and-forget global add (no value returned, so the thread does not wait for it).
@@ -372,11 +368,11 @@ __device__ __forceinline__ void griddep_launch_dependents() {
 }
 
 template <typename... P, typename... A>
-inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+inline cudaError_t launch_dep_smem(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -386,9 +382,20 @@ inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, cudaS
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+template <typename... P, typename... A>
+inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+    return launch_dep_smem(kernel, grid, block, 0, st, args...);
+}
+
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 

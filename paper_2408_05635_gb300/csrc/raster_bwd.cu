@@ -21,11 +21,10 @@
 // 8 x 4 patch of the tile and walks, back to front, only the staged Gaussians whose
 // footprint can reach alpha_min on the patch (build_patch_list) and that precede its last
 // contributor.
-// Reduction: every (pixel, Gaussian) term is summed over the warp with a butterfly
-// reduce-scatter (for the pose-only walk 6 values in 8 shuffles, or two Gaussians' 12 in
-// 13 when it steps two at a time; 16 values in 16 otherwise),
-// added by the owning lanes into a per-batch shared-memory accumulator, and flushed once
-// per (tile, Gaussian) with vector float4 atomics into the record's global accumulator.
+// Reduction: each warp sums its 32 pixels' terms of eight Gaussians at a time through a
+// small shared matrix read transposed (bwd_walk.cuh), adds the sums into a per-batch
+// shared-memory accumulator, and the block flushes once per (tile, Gaussian) with vector
+// float4 atomics into the record's global accumulator.
 // Lanes whose pixel the Gaussian does not reach take a = 0, which leaves T and g.B
 // unchanged and zeroes every term, so the walk has no divergent branch.
 #include "gs_internal.cuh"
@@ -33,26 +32,29 @@
 
 namespace gsk {
 
-// Shared accumulator slots per staged Gaussian: 0, 1 sum dp dx, dp dy; 2 sum a T g_D;
-// 3 sum dL/da a_raw; 4..6 sum dp dx^2, dp dx dy, dp dy^2; 8..10 sum a T g_C; 7, 11 unused.
-// POSE: only slots 0, 1, 2, 4, 5, 6 (what the pose gradient needs).
+// Four blocks per SM (64 registers a thread: the walk's unrolled steps spill at 48).
+// Dynamic shared memory: kWalkFloats per warp.
 template <bool POSE, int NB, int LW>
-__global__ void __launch_bounds__(kTilePix, 5) k_backward(BackwardLaunch L) {
+__global__ void __launch_bounds__(kTilePix, 4) k_backward(BackwardLaunch L) {
     static_assert(NB % 32 == 0 && NB <= kBatch, "batch depth: a multiple of 32, at most kBatch");
     static_assert(LW >= 3 && (1 << LW) * kPatchH <= kTilePix, "tile width: 8 to 32 pixels");
     griddep_wait();  // the predecessor's results are visible from here on
     griddep_launch_dependents();
-    __shared__ float4 sP0[NB], sC[NB], sQ[NB], sBox[NB];
+    using A = Acc<POSE>;
+    extern __shared__ __align__(16) float sDyn[];
+    __shared__ float4 sP0[NB], sC[NB], sBox[NB];
     __shared__ float4 sP1[NB];  // (kuu, lo, -1/(2 kuu), -1/(2 kvv)): the stride of sP0, sC
-    __shared__ float sAcc[NB * kAccStride];
-    __shared__ uint16_t sList[kTilePix / 32][NB];  // byte offsets: 16 x batch position
+    __shared__ float sAcc[NB * A::kStride];
+    __shared__ __align__(16) uint16_t sList[kTilePix / 32][NB];  // byte offsets: 16 x batch position
     __shared__ int s_view;
     __shared__ uint32_t s_nmax;
+    __shared__ unsigned long long s_count[2];
     const uint32_t tile = L.ws.tile_order[blockIdx.x];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
         s_view = view_of_tile(L.ws.views, L.d.V, tile);
         s_nmax = 0;
+        s_count[0] = s_count[1] = 0ull;
     }
     __syncthreads();
     const ViewInfo vi = L.ws.views[s_view];
@@ -69,26 +71,7 @@ __global__ void __launch_bounds__(kTilePix, 5) k_backward(BackwardLaunch L) {
     const float pv_lo = (float)pv0, pv_hi = (float)(pv0 + kPatchH - 1);
     const Settings &S = L.s;
     const float thr = S.log2_alpha_min;
-    // the accumulator slot this lane adds after a reduction, or -1
-    int my_slot = -1, pair_slot = -1;
-    if (POSE) {
-        // the paired steps' joint reduction: value 3 b3 + (b1 ? 2 : b2) of Gaussian b4
-        if ((lane & 1) == 0 && !((lane & 2) && (lane & 4))) {
-            const int k = ((lane & 8) ? 3 : 0) + ((lane & 2) ? 2 : ((lane & 4) ? 1 : 0));
-            pair_slot = k < 3 ? k : k + 1;  // values 0..5 -> slots 0, 1, 2, 4, 5, 6
-        }
-        if ((lane & 3) == 0 && !((lane & 8) && (lane & 4))) {
-            const int k = ((lane & 16) ? 3 : 0) + ((lane & 4) ? 2 : ((lane & 8) ? 1 : 0));
-            my_slot = k < 3 ? k : k + 1;  // values 0..5 -> slots 0, 1, 2, 4, 5, 6
-        }
-    } else {
-        int idx = 0;
-        if (lane & 16) idx += 8;
-        if (lane & 8) idx += 4;
-        if (lane & 4) idx += 2;
-        if (lane & 2) idx += 1;
-        if ((lane & 1) == 0 && idx != 7 && idx != 11 && idx < kAccStride) my_slot = idx;
-    }
+    float *buf = sDyn + warp * kWalkFloats<POSE>;
 
     uint32_t start;
     const uint32_t n = tile_entries(L.ws, L.d, tile, start);
@@ -115,6 +98,8 @@ __global__ void __launch_bounds__(kTilePix, 5) k_backward(BackwardLaunch L) {
     if (lane == 0 && wlast) atomicMax(&s_nmax, wlast);
     __syncthreads();
     const uint32_t nmax = s_nmax;
+    const PixUp up{g0, g1, g2, gD, gS};
+    store_planes<POSE>(buf, up, lane);
     float GB = 0.f;  // g . (colour, depth, 1) of everything behind, back-to-front
     uint32_t n_eval = 0, n_contrib = 0;
 
@@ -128,7 +113,6 @@ __global__ void __launch_bounds__(kTilePix, 5) k_backward(BackwardLaunch L) {
                 sP0[tid] = f.p0;
                 sP1[tid] = f.p1;
                 sC[tid] = make_float4(rr.c.x, rr.c.y, rr.c.z, rr.a.z);
-                sQ[tid] = make_float4(rr.b.x, rr.b.y, rr.b.z, rr.a.w);
                 sBox[tid] = stage_box(rr.b, -f.p0.x, -f.p0.y);
             } else {
                 sBox[tid] = make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY);
@@ -136,94 +120,49 @@ __global__ void __launch_bounds__(kTilePix, 5) k_backward(BackwardLaunch L) {
         }
         if (tid < NB) {  // thread tid owns the accumulator row of batch position tid
 #pragma unroll
-            for (int k = 0; k < kAccStride; ++k) sAcc[tid * kAccStride + k] = 0.f;
+            for (int k = 0; k < A::kValues; ++k) sAcc[tid * A::kStride + k] = 0.f;
         }
         __syncthreads();
         // this warp's list, limited to entries below its largest contributor count
         const int wcnt = (int)min((int64_t)cnt, (int64_t)wlast - b0);
         const int nl = build_patch_list(sBox, sP0, sP1, sList[warp], wcnt, lane, thr, pu_lo, pu_hi, pv_lo, pv_hi);
-        int e = nl - 1;
         // entries at byte offsets below lim are in front of this pixel's last contributor
         const int lim = (int)max(min((int64_t)last - b0, (int64_t)NB), (int64_t)0) * 16;
-        if constexpr (POSE) {
-            // two Gaussians per step: the pixel state is updated in depth order (the back
-            // one first), and the two reductions are independent, so they overlap
-            for (; e >= 1; e -= 2) {
-                const int jA = sList[warp][e], jB = sList[warp][e - 1];
-                const PolyEval pA = eval_poly(uv, at_off(sP0, jA), p1_at(sP1, jA));
-                const PolyEval pB = eval_poly(uv, at_off(sP0, jB), p1_at(sP1, jB));
-                const bool lA = jA < lim, lB = jB < lim;
-                n_eval += lA + lB;
-                const bool cA = lA && pA.poly >= thr, cB = lB && pB.poly >= thr;
-                if (!__any_sync(0xffffffffu, cA || cB)) continue;
-                n_contrib += cA + cB;
-                const float s2 = bwd_pair_reduce(cA, pA, at_off(sC, jA), cB, pB, at_off(sC, jB), g0, g1, g2, gD,
-                                                 gS, S.alpha_max, T, GB, lane);
-                if (pair_slot >= 0 && s2 != 0.f)
-                    atomicAdd(&sAcc[(((lane & 16) ? jB : jA) >> 4) * kAccStride + pair_slot], s2);
-            }
-        }
-        for (; e >= 0; --e) {
-            const int j = sList[warp][e];
-            const bool live = j < lim;
-            const PolyEval pe = eval_poly(uv, at_off(sP0, j), p1_at(sP1, j));
-            n_eval += live;
-            const bool c = live && pe.poly >= thr;
-            if (!__any_sync(0xffffffffu, c)) continue;
-            n_contrib += c;
-            if constexpr (POSE) {
-                float v[6];
-                moments6(bwd_step(c, pe, at_off(sC, j), g0, g1, g2, gD, gS, S.alpha_max, T, GB), v);
-                const float sum = warp_reduce_scatter6(v[0], v[1], v[2], v[3], v[4], v[5], lane);
-                if (my_slot >= 0 && sum != 0.f) atomicAdd(&sAcc[(j >> 4) * kAccStride + my_slot], sum);
-            } else {
-                const float araw = ex2_approx(pe.poly);
-                const float a = c ? fminf(S.alpha_max, araw) : 0.f;
-                if (c) T = T * __fdividef(1.f, 1.f - a);  // transmittance in front of this Gaussian
-                const float4 Cc = at_off(sC, j);
-                const float gv = fmaf(g0, Cc.x, fmaf(g1, Cc.y, fmaf(g2, Cc.z, fmaf(gD, Cc.w, gS))));
-                const float diff = gv - GB;
-                const float dalpha = T * diff;
-                GB = fmaf(a, diff, GB);
-                const float w = a * T;
-                const float dp = araw < S.alpha_max ? dalpha * a : 0.f;
-                const float dpx = dp * pe.d.x, dpy = dp * pe.d.y;
-                float vals[16] = {dpx,     dpy,     w * gD, c && araw < S.alpha_max ? dalpha * araw : 0.f,
-                                  dpx * pe.d.x, dpx * pe.d.y, dpy * pe.d.y, 0.f,
-                                  w * g0,  w * g1,  w * g2, 0.f, 0.f, 0.f, 0.f, 0.f};
-                int slot;
-                const float sum = warp_reduce_scatter<16>(vals, lane, slot);
-                if (my_slot >= 0 && sum != 0.f) atomicAdd(&sAcc[(j >> 4) * kAccStride + my_slot], sum);
-            }
-        }
+        bwd_walk_batch<POSE, true>(sList[warp], nl, lim, sP0, sP1, sC, uv, pu_lo, pv_lo, thr, S.alpha_max, up, T, GB,
+                                   buf, sAcc, lane, n_eval, n_contrib);
         __syncthreads();
         if (tid < cnt) {
             const uint32_t r = L.ws.sorted[start + (uint32_t)b0 + tid];
             if (r < rec_slots(L.d)) {
-                const float *m = sAcc + tid * kAccStride;
-                const float4 Q = sQ[tid];
-                const float4 v0 = make_float4(Q.x * m[0] + Q.y * m[1], Q.y * m[0] + Q.z * m[1], m[2],
-                                              POSE ? 0.f : m[3] / Q.w);
-                const float4 v1 = make_float4(-0.5f * m[4], -m[5], -0.5f * m[6], 0.f);
-                if (v0.x != 0.f || v0.y != 0.f || v0.z != 0.f || v0.w != 0.f) atomicAdd(&L.ws.rec_grad[r].g0, v0);
-                if (v1.x != 0.f || v1.y != 0.f || v1.z != 0.f) atomicAdd(&L.ws.rec_grad[r].g1, v1);
-                if constexpr (!POSE) {
-                    const float4 v2 = make_float4(m[8], m[9], m[10], 0.f);
-                    if (v2.x != 0.f || v2.y != 0.f || v2.z != 0.f) atomicAdd(&L.ws.rec_grad[r].g2, v2);
-                }
+                const float4 Q = L.ws.rec[r].b;  // conic
+                flush_acc<POSE>(sAcc + tid * A::kStride, Q, POSE ? 1.f : L.ws.rec[r].a.w, L.ws.rec_grad + r);
             }
         }
         __syncthreads();
     }
-    count_pairs(n_eval, n_contrib, &L.ws.hdr->bwd_evals, &L.ws.hdr->bwd_contrib);
+    count_warp(n_eval, n_contrib, s_count);
+    __syncthreads();
+    if (tid == 0) {
+        red_add64(&L.ws.hdr->bwd_evals, s_count[0]);
+        red_add64(&L.ws.hdr->bwd_contrib, s_count[1]);
+    }
+}
+
+// One block per tile, warp_floats floats of dynamic shared memory per warp.
+cudaError_t launch_tiles(void (*kernel)(BackwardLaunch), const BackwardLaunch &L, int warp_floats, cudaStream_t st) {
+    const uint32_t threads = tile_threads(L.d);
+    const size_t smem = (size_t)(threads / 32) * (size_t)warp_floats * sizeof(float);
+    // static and dynamic shared memory together may pass the 48 KB a kernel gets unasked
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return e != cudaSuccess ? e : launch_dep_smem(kernel, dim3(L.d.T), dim3(threads), smem, st, L);
 }
 
 template <int NB, int LW>
 cudaError_t launch_backward_nb(const BackwardLaunch &L, cudaStream_t st) {
     if (L.pose_only)
-        return launch_dep(k_backward<true, NB, LW>, dim3(L.d.T), dim3(tile_threads(L.d)), st, L);
+        return launch_tiles(k_backward<true, NB, LW>, L, kWalkFloats<true>, st);
     else
-        return launch_dep(k_backward<false, NB, LW>, dim3(L.d.T), dim3(tile_threads(L.d)), st, L);
+        return launch_tiles(k_backward<false, NB, LW>, L, kWalkFloats<false>, st);
 }
 
 template <int NB>

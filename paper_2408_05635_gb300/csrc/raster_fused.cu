@@ -7,11 +7,12 @@
 // footprint code, the same per-warp lists, the same reduce-scatter; see raster_fwd.cu and
 // raster_bwd.cu for the arithmetic), with three differences in how the work is laid out:
 //   - each pixel's upstream gradient, final transmittance and last contributor stay in
-//     registers between the walks (they are still written to the workspace, so a later
-//     gs_backward finds the same state as after k_forward);
+//     registers between the walks and are not written to the workspace (the pass consumes
+//     its gradients itself: a gs_backward after it is refused);
 //   - the batch the forward staged last is usually the one the reverse walk starts with
 //     (a tile's whole list when it holds at most one batch): it is not staged again, and
-//     each warp cuts the list it built for it in the forward instead of building another;
+//     each warp cuts the list it built for it in the forward instead of building another,
+//     and goes on from its forward to its reverse walk without waiting for the other warps;
 //   - a tile's reverse walk starts as soon as its own forward ends, so the tiles that end
 //     the forward (the longest lists, launched first) overlap the reverse walks of the
 //     others instead of leaving SMs idle before a second kernel.
@@ -28,14 +29,13 @@ __device__ __forceinline__ float sgnf(float x) { return (float)((x > 0.f) - (x <
 
 // Stage batch position tid of the tile's sorted list (record r) for both walks.
 __device__ __forceinline__ void stage_one(const TrackTileLaunch &L, uint32_t r, float x0, float y0, float4 *sP0,
-                                          float4 *sP1, float4 *sC, float4 *sQ, float4 *sBox, int tid) {
+                                          float4 *sP1, float4 *sC, float4 *sBox, int tid) {
     if (r < rec_slots(L.d)) {
         const Rec rr = L.ws.rec[r];
         const Footprint f = stage_footprint(rr.a, rr.b, x0, y0);
         sP0[tid] = f.p0;
         sP1[tid] = f.p1;
         sC[tid] = make_float4(rr.c.x, rr.c.y, rr.c.z, rr.a.z);
-        sQ[tid] = make_float4(rr.b.x, rr.b.y, rr.b.z, rr.a.w);
         sBox[tid] = stage_box(rr.b, -f.p0.x, -f.p0.y);
     } else {
         sBox[tid] = make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY);  // empty: never listed
@@ -44,8 +44,11 @@ __device__ __forceinline__ void stage_one(const TrackTileLaunch &L, uint32_t r, 
 
 }  // namespace
 
-constexpr int kFusedScratch = (2 * kSortSmemKeys * 8 > kBatch * kAccStride * 4) ? 2 * kSortSmemKeys * 8
-                                                                               : kBatch * kAccStride * 4;
+// One scratch of shared memory holds the sort's two key buffers, then each warp's
+// transposed rows of the reverse walk.
+constexpr int kFusedWarps = kTilePix / 32;
+constexpr int kFusedRows = kFusedWarps * kWalkFloats<true> * (int)sizeof(float);
+constexpr int kFusedScratch = 2 * kSortSmemKeys * 8 > kFusedRows ? 2 * kSortSmemKeys * 8 : kFusedRows;
 
 // Four blocks per SM (64 registers a thread): with five (48 registers) the walks spill
 // and issue more instructions, and the kernel is slower.
@@ -55,22 +58,24 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
     static_assert(LW >= 3 && (1 << LW) * kPatchH <= kTilePix, "tile width: 8 to 32 pixels");
     griddep_wait();  // the predecessor's results are visible from here on
     griddep_launch_dependents();
-    __shared__ float4 sP0[NB], sC[NB], sQ[NB], sBox[NB];
+    using A = Acc<true>;
+    __shared__ float4 sP0[NB], sC[NB], sBox[NB];
     __shared__ float4 sP1[NB];                     // (kuu, lo, -1/(2 kuu), -1/(2 kvv)): the stride of sP0, sC
-    __shared__ uint16_t sList[kTilePix / 32][NB];  // byte offsets: 16 x batch position
-    // the sort's two key buffers, then (reverse walk) the per-batch accumulators
+    __shared__ __align__(16) uint16_t sList[kTilePix / 32][NB];  // byte offsets: 16 x batch position
+    __shared__ float sAcc[NB * A::kStride];
     __shared__ __align__(16) unsigned char sScratch[kFusedScratch];
     unsigned long long *sKeys = reinterpret_cast<unsigned long long *>(sScratch);
-    float *sAcc = reinterpret_cast<float *>(sScratch);
     __shared__ int s_view;
     __shared__ float s_loss[kTilePix / 32];
     __shared__ uint32_t s_nmax;
+    __shared__ unsigned long long s_count[4];
     const uint32_t tile = L.ws.tile_order[blockIdx.x];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
         s_view = view_of_tile(L.ws.views, L.d.V, tile);
         s_nmax = 0;
     }
+    if (tid < 4) s_count[tid] = 0ull;
     __syncthreads();
     const ViewInfo vi = L.ws.views[s_view];
     const uint32_t local = tile - vi.tile_base;
@@ -110,8 +115,12 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
     for (uint32_t b0 = 0; b0 < n; b0 += NB) {
         if (__syncthreads_count(!walk.done) == 0) break;
         const uint32_t idx = b0 + tid;
-        if (tid < NB && idx < n) stage_one(L, L.ws.sorted[start + idx], x0, y0, sP0, sP1, sC, sQ, sBox, tid);
+        if (tid < NB && idx < n) stage_one(L, L.ws.sorted[start + idx], x0, y0, sP0, sP1, sC, sBox, tid);
         staged = b0;
+        if (b0 == 0 && tid < NB) {  // the reverse walk's sums (thread tid owns the row of batch position tid)
+#pragma unroll
+            for (int k = 0; k < A::kValues; ++k) sAcc[tid * A::kStride + k] = 0.f;
+        }
         __syncthreads();
         if (!targets_loaded) {
             targets_loaded = true;
@@ -137,7 +146,7 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
     const float cr = walk.cr, cg = walk.cg, cb = walk.cb, D = walk.D;
     uint32_t last = walk.last;
     const float Sil = 1.f - T;  // Eq. 4 summed: 1 - prod(1 - a_i)
-    count_pairs(n_eval, n_contrib, &L.ws.hdr->fwd_evals, &L.ws.hdr->fwd_contrib);
+    count_warp(n_eval, n_contrib, s_count);
 
     // ---------------------------------------------------------------- fused loss
     if (!targets_loaded && inside) {  // an empty tile list: no batch was staged
@@ -150,8 +159,6 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
     }
     float g0 = 0.f, g1 = 0.f, g2 = 0.f, gD = 0.f, gS = 0.f, l = 0.f;
     if (inside) {
-        L.ws.t_final[gp] = T;
-        L.ws.n_last[gp] = last;
         const bool valid = Dt > 0.f;
         const bool M = valid && Sil > S.sil_thresh;
         if (M) {
@@ -175,13 +182,6 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
             l += S.w_vis * (1.f - Sil);
             gS = -S.w_vis;
         }
-        const uint32_t P = L.d.P;
-        float *ug = L.ws.upstream + 3u * vi.pix_base;
-        ug[p] = g0;
-        ug[HW + p] = g1;
-        ug[2u * HW + p] = g2;
-        L.ws.upstream[3u * P + gp] = gD;
-        L.ws.upstream[4u * P + gp] = gS;
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
@@ -192,46 +192,38 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
     // the reverse walk evaluates this pixel's entries in front of its last contributor and
     // differentiates its contributions: the forward's counts up to that entry
     const uint32_t rev_eval = last ? walk.eval_last : 0u, rev_contrib = last ? n_contrib : 0u;
+    count_warp(rev_eval, rev_contrib, s_count + 2);
     uint32_t wlast = last;  // largest contributor count in the warp
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) wlast = max(wlast, __shfl_xor_sync(0xffffffffu, wlast, off));
     if (lane == 0 && wlast) atomicMax(&s_nmax, wlast);
-    __syncthreads();
-    if (tid == 0) {
-        DF s{0.f, 0.f};
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s = df_add(s, DF{s_loss[w], 0.f});
-        L.ws.tile_loss[tile] = df_pack(s);
-    }
-    const uint32_t nmax = s_nmax;
-    // the paired steps' joint reduction: value 3 b3 + (b1 ? 2 : b2) of Gaussian b4; the
-    // single steps': value 3 b4 + (b2 ? 2 : b3)
-    int my_slot = -1, pair_slot = -1;
-    if ((lane & 1) == 0 && !((lane & 2) && (lane & 4))) {
-        const int k = ((lane & 8) ? 3 : 0) + ((lane & 2) ? 2 : ((lane & 4) ? 1 : 0));
-        pair_slot = k < 3 ? k : k + 1;  // values 0..5 -> slots 0, 1, 2, 4, 5, 6
-    }
-    if ((lane & 3) == 0 && !((lane & 8) && (lane & 4))) {
-        const int k = ((lane & 16) ? 3 : 0) + ((lane & 4) ? 2 : ((lane & 8) ? 1 : 0));
-        my_slot = k < 3 ? k : k + 1;
-    }
+    const PixUp up{g0, g1, g2, gD, gS};
+    float *buf = reinterpret_cast<float *>(sScratch) + warp * kWalkFloats<true>;
+    store_planes<true>(buf, up, lane);
     float GB = 0.f;  // g . (colour, depth, 1) of everything behind, back-to-front
-    for (int64_t b0 = nmax ? (int64_t)((nmax - 1) / NB) * NB : -1; b0 >= 0; b0 -= NB) {
-        const int cnt = (int)min((uint32_t)NB, nmax - (uint32_t)b0);
-        if (b0 != staged && tid < cnt)
-            stage_one(L, L.ws.sorted[start + (uint32_t)b0 + tid], x0, y0, sP0, sP1, sC, sQ, sBox, tid);
-        if (tid < NB) {  // thread tid owns the accumulator row of batch position tid
+    // From the batch the forward staged last down to the first.  The staged one needs no
+    // barrier: each warp goes on from its forward to its reverse walk by itself, so the
+    // warps of a tile wait for one another once (before the flush) instead of after each walk.
+    for (int64_t b0 = staged; b0 >= 0; b0 -= NB) {
+        const bool resident = b0 == staged;
+        const uint32_t filled = min((uint32_t)NB, n - (uint32_t)b0);
+        if (!resident) {
+            __syncthreads();  // the flush of the batch behind has read the sums
+            if (tid < filled) stage_one(L, L.ws.sorted[start + (uint32_t)b0 + tid], x0, y0, sP0, sP1, sC, sBox, tid);
+            if (tid < NB) {
 #pragma unroll
-            for (int k = 0; k < kAccStride; ++k) sAcc[tid * kAccStride + k] = 0.f;
+                for (int k = 0; k < A::kValues; ++k) sAcc[tid * A::kStride + k] = 0.f;
+            }
+            __syncthreads();
         }
-        __syncthreads();
         // this warp's list, limited to entries below its largest contributor count
-        const int wcnt = (int)min((int64_t)cnt, (int64_t)wlast - b0);
+        const int wcnt = (int)max(min((int64_t)filled, (int64_t)wlast - b0), (int64_t)0);
         int nl = 0;
-        if (b0 == staged) {
-            // the batch the forward ended on: its list (ascending positions) is still in
-            // sList, and the entries below wcnt are the list build_patch_list would give for
-            // wcnt.  A warp whose pixels had all stopped before this batch kept an older
-            // list, but then wlast <= b0 and no entry is below wcnt <= 0.
+        if (resident) {
+            // the list this warp built for the batch in the forward is still in sList, and
+            // its entries below wcnt are the list build_patch_list would give for wcnt.  A
+            // warp whose pixels had all stopped before this batch kept an older list, but
+            // then wlast <= b0 and no entry is below wcnt = 0.
             for (int k = 0; k < nl_staged; k += 32) {
                 const bool below = k + lane < nl_staged && (int)sList[warp][k + lane] < wcnt * 16;
                 const int m = __popc(__ballot_sync(0xffffffffu, below));
@@ -241,48 +233,29 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
         } else {
             nl = build_patch_list(sBox, sP0, sP1, sList[warp], wcnt, lane, thr, pu_lo, pu_hi, pv_lo, pv_hi);
         }
-        int e = nl - 1;
+        __syncwarp();
         // entries at byte offsets below lim are in front of this pixel's last contributor
         const int lim = (int)max(min((int64_t)last - b0, (int64_t)NB), (int64_t)0) * 16;
-        // two Gaussians per step: the pixel state is updated in depth order (the back one
-        // first), and the two reductions are independent, so they overlap
-        for (; e >= 1; e -= 2) {
-            const int jA = sList[warp][e], jB = sList[warp][e - 1];
-            const PolyEval pA = eval_poly(uv, at_off(sP0, jA), p1_at(sP1, jA));
-            const PolyEval pB = eval_poly(uv, at_off(sP0, jB), p1_at(sP1, jB));
-            const bool cA = jA < lim && pA.poly >= thr, cB = jB < lim && pB.poly >= thr;
-            if (!__any_sync(0xffffffffu, cA || cB)) continue;
-            const float s2 = bwd_pair_reduce(cA, pA, at_off(sC, jA), cB, pB, at_off(sC, jB), g0, g1, g2, gD, gS,
-                                             S.alpha_max, T, GB, lane);
-            if (pair_slot >= 0 && s2 != 0.f)
-                atomicAdd(&sAcc[(((lane & 16) ? jB : jA) >> 4) * kAccStride + pair_slot], s2);
-        }
-        for (; e >= 0; --e) {
-            const int j = sList[warp][e];
-            const PolyEval pe = eval_poly(uv, at_off(sP0, j), p1_at(sP1, j));
-            const bool c = j < lim && pe.poly >= thr;
-            if (!__any_sync(0xffffffffu, c)) continue;
-            float v[6];
-            moments6(bwd_step(c, pe, at_off(sC, j), g0, g1, g2, gD, gS, S.alpha_max, T, GB), v);
-            const float sum = warp_reduce_scatter6(v[0], v[1], v[2], v[3], v[4], v[5], lane);
-            if (my_slot >= 0 && sum != 0.f) atomicAdd(&sAcc[(j >> 4) * kAccStride + my_slot], sum);
-        }
+        uint32_t unused = 0;
+        bwd_walk_batch<true, false>(sList[warp], nl, lim, sP0, sP1, sC, uv, pu_lo, pv_lo, thr, S.alpha_max, up, T, GB,
+                                    buf, sAcc, lane, unused, unused);
         __syncthreads();
-        if (tid < cnt) {
+        const uint32_t nmax = s_nmax;
+        if (nmax > (uint32_t)b0 && tid < min(filled, nmax - (uint32_t)b0)) {
             const uint32_t r = L.ws.sorted[start + (uint32_t)b0 + tid];
-            if (r < rec_slots(L.d)) {
-                const float *m = sAcc + tid * kAccStride;
-                const float4 Q = sQ[tid];
-                const float4 v0 = make_float4(Q.x * m[0] + Q.y * m[1], Q.y * m[0] + Q.z * m[1], m[2], 0.f);
-                const float4 v1 = make_float4(-0.5f * m[4], -m[5], -0.5f * m[6], 0.f);
-                if (v0.x != 0.f || v0.y != 0.f || v0.z != 0.f) atomicAdd(&L.ws.rec_grad[r].g0, v0);
-                if (v1.x != 0.f || v1.y != 0.f || v1.z != 0.f) atomicAdd(&L.ws.rec_grad[r].g1, v1);
-            }
+            if (r < rec_slots(L.d)) flush_acc<true>(sAcc + tid * A::kStride, L.ws.rec[r].b, 1.f, L.ws.rec_grad + r);
         }
-        __syncthreads();
-        staged = -1;  // every later batch is staged again
     }
-    count_pairs(rev_eval, rev_contrib, &L.ws.hdr->bwd_evals, &L.ws.hdr->bwd_contrib);
+    if (staged < 0) __syncthreads();  // an empty list: the barrier before the flush did not run
+    if (tid == 0) {
+        DF s{0.f, 0.f};
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s = df_add(s, DF{s_loss[w], 0.f});
+        L.ws.tile_loss[tile] = df_pack(s);
+        red_add64(&L.ws.hdr->fwd_evals, s_count[0]);
+        red_add64(&L.ws.hdr->fwd_contrib, s_count[1]);
+        red_add64(&L.ws.hdr->bwd_evals, s_count[2]);
+        red_add64(&L.ws.hdr->bwd_contrib, s_count[3]);
+    }
 }
 
 template <int NB, int LW>

@@ -36,13 +36,17 @@ __global__ void __launch_bounds__(kTilePix, 5) k_forward(ForwardLaunch L) {
     griddep_launch_dependents();
     __shared__ float4 sP0[NB], sC[NB], sBox[NB];
     __shared__ float4 sP1[NB];                     // (kuu, lo, -1/(2 kuu), -1/(2 kvv)): the stride of sP0, sC
-    __shared__ uint16_t sList[kTilePix / 32][NB];  // byte offsets: 16 x batch position
+    __shared__ __align__(16) uint16_t sList[kTilePix / 32][NB];  // byte offsets: 16 x batch position
     __shared__ unsigned long long sKeys[2 * kSortSmemKeys];  // the sort's two buffers
     __shared__ int s_view;
     __shared__ float s_loss[kTilePix / 32];
+    __shared__ unsigned long long s_count[2];
     const uint32_t tile = L.ws.tile_order[blockIdx.x];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) s_view = view_of_tile(L.ws.views, L.d.V, tile);
+    if (tid == 0) {
+        s_view = view_of_tile(L.ws.views, L.d.V, tile);
+        s_count[0] = s_count[1] = 0ull;
+    }
     __syncthreads();
     const int view = s_view;
     (void)view;
@@ -118,7 +122,7 @@ __global__ void __launch_bounds__(kTilePix, 5) k_forward(ForwardLaunch L) {
     const float T = walk.T, cr = walk.cr, cg = walk.cg, cb = walk.cb, D = walk.D;
     const uint32_t last = walk.last;
     const float Sil = 1.f - T;
-    count_pairs(n_eval, n_contrib, &L.ws.hdr->fwd_evals, &L.ws.hdr->fwd_contrib);
+    count_warp(n_eval, n_contrib, s_count);
 
     if (inside) {
         if (L.rgb) {
@@ -174,12 +178,16 @@ __global__ void __launch_bounds__(kTilePix, 5) k_forward(ForwardLaunch L) {
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
         if ((tid & 31) == 0) s_loss[tid >> 5] = l;
-        __syncthreads();
-        if (tid == 0) {
+    }
+    __syncthreads();
+    if (tid == 0) {
+        if constexpr (LOSS) {
             DF s{0.f, 0.f};
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s = df_add(s, DF{s_loss[w], 0.f});
             L.ws.tile_loss[tile] = df_pack(s);
         }
+        red_add64(&L.ws.hdr->fwd_evals, s_count[0]);
+        red_add64(&L.ws.hdr->fwd_contrib, s_count[1]);
     }
 }
 
