@@ -6,8 +6,12 @@
 // All three are HBM-bound passes over flat arrays.  The two that change the number of
 // Gaussians are stable compactions in two launches: a block-count pass, then an emit
 // pass in which every block sums the counts of the blocks before it (at most a few
-// thousand words, read from L2) and scatters its items in order.  No block waits on
-// another, and the live count stays on the device.
+// thousand words, read from L2) and writes its items in order.  A block's items are one
+// contiguous run of rows in every output array, so it writes each array value by value
+// (consecutive threads, consecutive words) instead of a row of three or four values per
+// thread: at 1M Gaussians with moments and an FP16 copy k_prune_emit takes 73 us against 108
+// (425 MB: 63 us at the copy rate), and for 154 k new Gaussians of a 640 x 480 frame
+// k_add_emit 19 us against 44 (part of that was FP64, below).  No block waits on another, and the live count stays on the device.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -65,13 +69,6 @@ __device__ __forceinline__ void store_lowp(void *base, int64_t i, float x, int d
         static_cast<__half *>(base)[i] = __float2half_rn(x);
 }
 
-__device__ __forceinline__ void copy_lowp(const void *src, int64_t i, void *dst, int64_t j, int dt) {
-    if (dt == GS_BF16)
-        static_cast<__nv_bfloat16 *>(dst)[j] = static_cast<const __nv_bfloat16 *>(src)[i];
-    else
-        static_cast<__half *>(dst)[j] = static_cast<const __half *>(src)[i];
-}
-
 // Sum of counts[0, b) over the block, and the total when b is the last block.
 __device__ uint32_t block_prefix(const uint32_t *counts, uint32_t b) {
     __shared__ uint32_t s_w[kCompactThreads / 32];
@@ -113,6 +110,56 @@ __device__ uint32_t block_rank(bool flag, uint32_t &count) {
 
 // ------------------------------------------------------------------ new Gaussians
 
+// FP32 pairs (hi + lo): the FP64 values of the camera that the unprojection takes, and its
+// arithmetic.  FP64 issues at a sixty-fourth of the FP32 rate here and bound the pass; pairs
+// keep about 2^-45, so the FP32 means and log-scales round as from FP64 but for near ties.
+using gsk::DF;
+using gsk::df_add;
+
+DF df_host(double x) {
+    const float hi = (float)x;
+    return DF{hi, std::isfinite(hi) ? (float)(x - (double)hi) : 0.f};
+}
+__device__ __forceinline__ DF df_split(double x) {
+    const float hi = (float)x;
+    return DF{hi, (float)(x - (double)hi)};
+}
+__device__ __forceinline__ DF df_mul(DF a, DF b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    const float e = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.hi, -p)));
+    const float s = __fadd_rn(p, e);
+    return DF{s, __fsub_rn(e, __fsub_rn(s, p))};
+}
+
+// ln x, rounded to FP32 from about 30 bits: x = 2^k m, m in [sqrt(1/2), sqrt(2)),
+// ln m = 2 atanh(s) = 2 (s + s^3 / 3 + ... + s^13 / 13), s = (m - 1) / (m + 1), |s| < 0.172 (the
+// next term is below 2e-12 of s); s and k ln 2 as pairs, the rest of the series, at most
+// 1 % of s, in FP32.  x: a positive normal pair.
+constexpr double kLn2 = 0.69314718055994530942;
+constexpr float kLn2Hi = 90852.f / 131072.f;  // 17 bits: k kLn2Hi is exact
+constexpr float kLn2Lo = (float)(kLn2 - (double)kLn2Hi);
+
+__device__ __forceinline__ float log_pair(DF x) {
+    const int bits = __float_as_int(x.hi), k = (bits - __float_as_int(0.70710678f)) >> 23;
+    const float mh = __int_as_float(bits - (k << 23)), ml = ldexpf(x.lo, -k);
+    const DF num = df_add(DF{__fsub_rn(mh, 1.f), 0.f}, DF{ml, 0.f});  // mh - 1 is exact
+    const DF den = df_add(DF{mh, ml}, DF{1.f, 0.f});
+    const float q = __fdiv_rn(num.hi, den.hi);
+    const float r = __fadd_rn(__fmaf_rn(-q, den.hi, num.hi), __fmaf_rn(-q, den.lo, num.lo));
+    const DF s = DF{q, __fdiv_rn(r, den.hi)};
+    const float z = q * q;
+    float t = 1.f / 13.f;
+    t = fmaf(t, z, 1.f / 11.f);
+    t = fmaf(t, z, 1.f / 9.f);
+    t = fmaf(t, z, 1.f / 7.f);
+    t = fmaf(t, z, 1.f / 5.f);
+    t = fmaf(t, z, 1.f / 3.f);
+    const float fk = (float)k;
+    DF sum = df_add(DF{fk * kLn2Hi, fk * kLn2Lo}, DF{2.f * s.hi, 2.f * s.lo});
+    sum = df_add(sum, DF{2.f * q * (z * t), 0.f});
+    return sum.hi;
+}
+
 struct AddLaunch {
     MapView map;
     int64_t *n;
@@ -120,9 +167,11 @@ struct AddLaunch {
     const float *rgb, *depth, *sil;
     float sil_add;
     double fx, fy, cx, cy;
+    DF ifx, ify, ncx, ncy, inv_f;  // 1 / fx, 1 / fy, -cx, -cy, 2 / (fx + fy)
     int32_t width, height;
     uint32_t *counts;  // scratch: one word per block
     int64_t *n0;       // scratch: the live count before the call
+    double *Rt;        // scratch: world->camera rotation (9) and translation (3)
     uint32_t *err;
 };
 
@@ -140,74 +189,104 @@ __global__ void __launch_bounds__(kCompactThreads) k_add_count(AddLaunch L) {
         L.counts[blockIdx.x] = c;
         if (blockIdx.x == 0) *L.n0 = *L.n;
     }
-}
-
-__global__ void __launch_bounds__(kCompactThreads) k_add_emit(AddLaunch L) {
-    __shared__ double s_R[9], s_t[3];
-    const int64_t P = (int64_t)L.width * L.height;
-    const int64_t p = (int64_t)blockIdx.x * kCompactThreads + threadIdx.x;
-    if (threadIdx.x == 0) {
-        // world->camera rotation of the pose's unit quaternion (renormalised), in FP64
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 32) {
+        // the rotation of the pose's unit quaternion (renormalised), in FP64: once here
+        // instead of in front of every block of the emission
         double w = L.pose[0], x = L.pose[1], y = L.pose[2], z = L.pose[3];
         const double inv = 1.0 / sqrt(w * w + x * x + y * y + z * z);
         w *= inv; x *= inv; y *= inv; z *= inv;
-        s_R[0] = 1.0 - 2.0 * (y * y + z * z); s_R[1] = 2.0 * (x * y - w * z); s_R[2] = 2.0 * (x * z + w * y);
-        s_R[3] = 2.0 * (x * y + w * z); s_R[4] = 1.0 - 2.0 * (x * x + z * z); s_R[5] = 2.0 * (y * z - w * x);
-        s_R[6] = 2.0 * (x * z - w * y); s_R[7] = 2.0 * (y * z + w * x); s_R[8] = 1.0 - 2.0 * (x * x + y * y);
-        s_t[0] = L.pose[4]; s_t[1] = L.pose[5]; s_t[2] = L.pose[6];
+        double *R = L.Rt;
+        R[0] = 1.0 - 2.0 * (y * y + z * z); R[1] = 2.0 * (x * y - w * z); R[2] = 2.0 * (x * z + w * y);
+        R[3] = 2.0 * (x * y + w * z); R[4] = 1.0 - 2.0 * (x * x + z * z); R[5] = 2.0 * (y * z - w * x);
+        R[6] = 2.0 * (x * z - w * y); R[7] = 2.0 * (y * z + w * x); R[8] = 1.0 - 2.0 * (x * x + y * y);
+        R[9] = L.pose[4]; R[10] = L.pose[5]; R[11] = L.pose[6];
     }
+}
+
+// The pixel's sample point at depth d in the camera frame (inverse of pi_m), then
+// world = R^T (x_c - t), and the log-scale ln(d / f): in FP64, for depths whose pairs would
+// leave FP32's range.
+__device__ __noinline__ void unproject_fp64(const AddLaunch &L, const double *R, const double *t, int u, int v, double d,
+                                            float (&mean)[3], float &ls) {
+    const double xc0 = ((double)u - L.cx) / L.fx * d - t[0];
+    const double xc1 = ((double)v - L.cy) / L.fy * d - t[1];
+    const double xc2 = d - t[2];
+    for (int k = 0; k < 3; ++k) mean[k] = (float)(R[k] * xc0 + R[3 + k] * xc1 + R[6 + k] * xc2);
+    ls = (float)log(d / (0.5 * (L.fx + L.fy)));
+}
+
+// `values` consecutive values of one output array, value(i) the i-th; consecutive threads
+// take consecutive values.
+template <class T, class F>
+__device__ __forceinline__ void write_run(T *out, int values, F &&value) {
+    for (int i = threadIdx.x; i < values; i += kCompactThreads) out[i] = value(i);
+}
+template <class F>
+__device__ __forceinline__ void write_lowp(void *base, int64_t first, int values, int dt, F &&value) {
+    for (int i = threadIdx.x; i < values; i += kCompactThreads) store_lowp(base, first + i, value(i), dt);
+}
+
+// Two blocks per SM (32 registers): the block's phases wait for one another, so a second
+// block hides them (21 -> 19 us).
+__global__ void __launch_bounds__(kCompactThreads, 2) k_add_emit(AddLaunch L) {
+    __shared__ DF s_R[9], s_nt[3];  // R, -t
+    __shared__ float s_mean[3 * kCompactThreads], s_rgb[3 * kCompactThreads], s_ls[kCompactThreads];
+    const int64_t P = (int64_t)L.width * L.height;
+    const int64_t p = (int64_t)blockIdx.x * kCompactThreads + threadIdx.x;
+    if (threadIdx.x < 9) s_R[threadIdx.x] = df_split(L.Rt[threadIdx.x]);
+    else if (threadIdx.x < 12) s_nt[threadIdx.x - 9] = df_split(-L.Rt[threadIdx.x]);
     const uint32_t before = block_prefix(L.counts, blockIdx.x);
     const bool flag = add_flag(L, p, P);
     uint32_t count;
-    const uint32_t r = block_rank(flag, count);
-    const int64_t n0 = *L.n0;
-    const int64_t i = n0 + before + r;
+    const uint32_t r = block_rank(flag, count);  // (ends with a barrier: s_R and s_nt are set)
+    if (flag) {
+        const int v = (int)(p / L.width), u = (int)(p - (int64_t)v * L.width);
+        const float d = L.depth[p];
+        float mean[3], ls;
+        if (d > 0x1p-60f && d < 0x1p60f) {
+            const DF D{d, 0.f};
+            const DF x0 = df_add(df_mul(df_mul(df_add(DF{(float)u, 0.f}, L.ncx), L.ifx), D), s_nt[0]);
+            const DF x1 = df_add(df_mul(df_mul(df_add(DF{(float)v, 0.f}, L.ncy), L.ify), D), s_nt[1]);
+            const DF x2 = df_add(D, s_nt[2]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                mean[k] = df_add(df_add(df_mul(s_R[k], x0), df_mul(s_R[3 + k], x1)), df_mul(s_R[6 + k], x2)).hi;
+            ls = log_pair(df_mul(D, L.inv_f));
+        } else {
+            unproject_fp64(L, L.Rt, L.Rt + 9, u, v, (double)d, mean, ls);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            s_mean[3 * r + k] = mean[k];
+            s_rgb[3 * r + k] = L.rgb[k * P + p];
+        }
+        s_ls[r] = ls;
+    }
+    __syncthreads();
     const MapView &M = L.map;
-    if (flag && i < M.cap) {
-        const int64_t v = p / L.width, u = p - v * L.width;
-        const double d = (double)L.depth[p];
-        // the pixel's sample point at depth d in the camera frame (inverse of pi_m), then
-        // world = R^T (x_c - t)
-        const double xc0 = ((double)u - L.cx) / L.fx * d - s_t[0];
-        const double xc1 = ((double)v - L.cy) / L.fy * d - s_t[1];
-        const double xc2 = d - s_t[2];
+    const int64_t n0 = *L.n0, first = n0 + before;
+    // the block's rows that fit the capacity
+    const int rows = first < M.cap ? (int)min((int64_t)count, M.cap - first) : 0;
+    const int wl = M.iso ? 1 : 3;
+    write_run(M.p[0] + 3 * first, 3 * rows, [&](int i) { return s_mean[i]; });
+    if (!M.iso) write_run(M.p[1] + 4 * first, 4 * rows, [&](int i) { return (i & 3) == 0 ? 1.f : 0.f; });
+    write_run(M.p[2] + wl * first, wl * rows, [&](int i) { return s_ls[wl == 1 ? i : i / 3]; });
+    write_run(M.p[3] + first, rows, [&](int) { return 0.f; });
+    write_run(M.p[4] + 3 * first, 3 * rows, [&](int i) { return s_rgb[i]; });
+    if (M.lp[2]) {
+        const int dt = M.lowp_dt;
+        if (M.lp[1]) write_lowp(M.lp[1], 4 * first, 4 * rows, dt, [&](int i) { return (i & 3) == 0 ? 1.f : 0.f; });
+        write_lowp(M.lp[2], wl * first, wl * rows, dt, [&](int i) { return s_ls[wl == 1 ? i : i / 3]; });
+        write_lowp(M.lp[3], first, rows, dt, [&](int) { return 0.f; });
+        write_lowp(M.lp[4], 3 * first, 3 * rows, dt, [&](int i) { return s_rgb[i]; });
+    }
+    if (M.state) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k)
-            M.p[0][3 * i + k] = (float)(s_R[k] * xc0 + s_R[3 + k] * xc1 + s_R[6 + k] * xc2);
-        const float ls = (float)log(d / (0.5 * (L.fx + L.fy)));
-        const float q[4] = {1.f, 0.f, 0.f, 0.f};
-        const float c[3] = {L.rgb[p], L.rgb[P + p], L.rgb[2 * P + p]};
-        const int wl = group_width(2, M.iso);
-        if (!M.iso) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) M.p[1][4 * i + k] = q[k];
-        }
-        for (int k = 0; k < wl; ++k) M.p[2][wl * i + k] = ls;
-        M.p[3][i] = 0.f;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) M.p[4][3 * i + k] = c[k];
-        if (M.lp[2]) {
-            if (M.lp[1]) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) store_lowp(M.lp[1], 4 * i + k, q[k], M.lowp_dt);
-            }
-            for (int k = 0; k < wl; ++k) store_lowp(M.lp[2], wl * i + k, ls, M.lowp_dt);
-            store_lowp(M.lp[3], i, 0.f, M.lowp_dt);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) store_lowp(M.lp[4], 3 * i + k, c[k], M.lowp_dt);
-        }
-        if (M.state) {
-            const int vp = values_per_gaussian(M.iso);
-#pragma unroll
-            for (int s = 0; s < kGroups; ++s) {
-                const int w = group_width(s, M.iso);
-                float *m = M.state + M.cap * group_offset(s, M.iso);
-                float *vv = m + vp * M.cap;
-                for (int k = 0; k < w; ++k) {
-                    m[w * i + k] = 0.f;
-                    vv[w * i + k] = 0.f;
-                }
-            }
+        for (int s = 0; s < kGroups; ++s) {
+            const int w = group_width(s, M.iso);
+            float *m = M.state + M.cap * group_offset(s, M.iso) + w * first;
+            write_run(m, w * rows, [&](int) { return 0.f; });
+            write_run(m + values_per_gaussian(M.iso) * M.cap, w * rows, [&](int) { return 0.f; });
         }
     }
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
@@ -310,39 +389,71 @@ __global__ void __launch_bounds__(kCompactThreads) k_prune_count(PruneLaunch L) 
     }
 }
 
+// One group of values (S) of a block's kept Gaussians: row r of the destination's rows
+// [j0, j0 + count) is row i0 + idx[r] of the source, in the parameters, the low-precision
+// copy (16-bit values, moved as they are) and both moments.  A thread takes W values of each
+// array, all their loads before the first store: at four loads in flight the pass was bound
+// by latency (137 us at 1.2M Gaussians).
+template <int S, bool ISO>
+__device__ __forceinline__ void prune_group(const PruneLaunch &L, int64_t i0, int64_t j0, const uint16_t *idx, int count) {
+    constexpr int W = group_width(S, ISO);
+    if constexpr (W > 0) {
+        const MapView &A = L.src, &B = L.dst;
+        const bool lowp = S > 0 && A.lp[S] && B.lp[S] && A.lowp_dt == B.lowp_dt, state = A.state && B.state;
+        constexpr int64_t o = group_offset(S, ISO), vp = values_per_gaussian(ISO);
+        const float *sp = A.p[S] + W * i0, *sm = A.state + A.cap * o + W * i0, *sv = sm + vp * A.cap;
+        float *dp = B.p[S] + W * j0, *dm = B.state + B.cap * o + W * j0, *dv = dm + vp * B.cap;
+        const uint16_t *sl = static_cast<const uint16_t *>(A.lp[S]) + W * i0;
+        uint16_t *dl = static_cast<uint16_t *>(B.lp[S]) + W * j0;
+        float p[W], m[W], v[W];
+        uint16_t l[W];
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            const int i = threadIdx.x + k * kCompactThreads, r = i / W;
+            if (i < W * count) {
+                const int at = W * (int)idx[r] + (i - W * r);
+                p[k] = sp[at];
+                if (state) m[k] = sm[at];
+                if (state) v[k] = sv[at];
+                if (lowp) l[k] = sl[at];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            const int i = threadIdx.x + k * kCompactThreads;
+            if (i < W * count) {
+                dp[i] = p[k];
+                if (state) dm[i] = m[k];
+                if (state) dv[i] = v[k];
+                if (lowp) dl[i] = l[k];
+            }
+        }
+    }
+}
+
+template <bool ISO>
 __global__ void __launch_bounds__(kCompactThreads) k_prune_emit(PruneLaunch L) {
-    const int64_t i = (int64_t)blockIdx.x * kCompactThreads + threadIdx.x;
+    __shared__ uint16_t s_idx[kCompactThreads];
+    const int64_t i0 = (int64_t)blockIdx.x * kCompactThreads, i = i0 + threadIdx.x;
     const int64_t n = *L.n0;
     const uint32_t before = block_prefix(L.counts, blockIdx.x);
     const bool keep = i < n && L.src.p[3][i] >= L.logit_min;
     uint32_t count;
     const uint32_t r = block_rank(keep, count);
-    const MapView &S = L.src, &D = L.dst;
-    if (keep) {
-        const int64_t j = (int64_t)before + r;
-        const int vp = values_per_gaussian(S.iso);
-#pragma unroll
-        for (int s = 0; s < kGroups; ++s) {
-            const int w = group_width(s, S.iso);
-            for (int k = 0; k < w; ++k) D.p[s][w * j + k] = S.p[s][w * i + k];
-            if (s > 0 && S.lp[s] && D.lp[s] && S.lowp_dt == D.lowp_dt)
-                for (int k = 0; k < w; ++k) copy_lowp(S.lp[s], w * i + k, D.lp[s], w * j + k, D.lowp_dt);
-            if (S.state && D.state) {
-                const float *sm = S.state + S.cap * group_offset(s, S.iso);
-                float *dm = D.state + D.cap * group_offset(s, S.iso);
-                for (int k = 0; k < w; ++k) {
-                    dm[w * j + k] = sm[w * i + k];
-                    dm[vp * D.cap + w * j + k] = sm[vp * S.cap + w * i + k];
-                }
-            }
-        }
-    }
+    if (keep) s_idx[r] = (uint16_t)threadIdx.x;
+    __syncthreads();
+    const int64_t j0 = before;
+    prune_group<0, ISO>(L, i0, j0, s_idx, (int)count);
+    prune_group<1, ISO>(L, i0, j0, s_idx, (int)count);
+    prune_group<2, ISO>(L, i0, j0, s_idx, (int)count);
+    prune_group<3, ISO>(L, i0, j0, s_idx, (int)count);
+    prune_group<4, ISO>(L, i0, j0, s_idx, (int)count);
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *L.n_dst = (int64_t)before + count;
 }
 
 // ------------------------------------------------------------------ host side
 
-constexpr size_t kScratchHead = 256;  // the saved live count, then one word per block
+constexpr size_t kScratchHead = 256;  // the saved live count and the pose, then one word per block
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -410,9 +521,15 @@ gs_status gs_map_add(const gs_map_config *cfg, const gs_map *map, int64_t *n, co
     L.fy = cam->fy;
     L.cx = cam->cx;
     L.cy = cam->cy;
+    L.ifx = df_host(1.0 / cam->fx);
+    L.ify = df_host(1.0 / cam->fy);
+    L.ncx = df_host(-cam->cx);
+    L.ncy = df_host(-cam->cy);
+    L.inv_f = df_host(2.0 / (cam->fx + cam->fy));
     L.width = cam->width;
     L.height = cam->height;
     L.n0 = static_cast<int64_t *>(scratch);
+    L.Rt = static_cast<double *>(scratch) + 1;  // 96 bytes of the head
     L.counts = reinterpret_cast<uint32_t *>(static_cast<char *>(scratch) + kScratchHead);
     L.err = err_flags;
     const unsigned blocks = (unsigned)((P + kCompactThreads - 1) / kCompactThreads);
@@ -483,7 +600,8 @@ gs_status gs_map_prune(const gs_map_config *cfg, const gs_map *src, const int64_
     const unsigned blocks = (unsigned)std::max<int64_t>(1, (src->capacity + kCompactThreads - 1) / kCompactThreads);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     k_prune_count<<<blocks, kCompactThreads, 0, st>>>(L);
-    k_prune_emit<<<blocks, kCompactThreads, 0, st>>>(L);
+    if (L.src.iso) k_prune_emit<true><<<blocks, kCompactThreads, 0, st>>>(L);
+    else k_prune_emit<false><<<blocks, kCompactThreads, 0, st>>>(L);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
