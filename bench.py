@@ -966,7 +966,8 @@ def main():
     sch = R.schedule
     tiles = -(-cam.width // sch["tile_w"]) * -(-cam.height // sch["tile_h"])
     radix = 3 * gs.radix_passes(tiles) + 1 if sch["flags"] & gs.GS_SCHED_RADIX else 0  # passes x 3 + ties
-    per_iter_launches = 1 + 3 + radix + (1 if sch["flags"] & gs.GS_SCHED_FUSED else 2) + 2
+    sort = radix or 1  # the per-tile sort is one kernel
+    per_iter_launches = 1 + 3 + sort + (1 if sch["flags"] & gs.GS_SCHED_FUSED else 2) + 2
     if world > 1:
         dist.barrier()
     torch.cuda.synchronize(dev)

@@ -331,7 +331,7 @@ typedef struct {
 /* gs_schedule.flags: GS_SCHED_RADIX -- the front-to-back order of Eqs. 2-4 comes from one
  * device-wide LSD radix sort of all (tile, depth) keys (eight-bit digits, stable passes,
  * runs of equal keys then put in Gaussian order) run after the key emission, instead of
- * the per-tile sort inside the forward.  Same order, same results. */
+ * the per-tile sort before the forward.  Same order, same results. */
 #define GS_SCHED_RADIX 2
 
 /* Read the context's schedule (defaults after gs_create).  Errors: INVALID_ARG (NULL). */

@@ -5,8 +5,8 @@
 //               visible records, per-tile pair counts.
 //   k_scan_tiles  tile offsets, tile launch order (longest lists first).
 //   k_emit      visible record: one 64-bit key (depth bits << 32 | record) per tile met.
-//   k_forward   tile: sort its keys by (depth, Gaussian index), then Eqs. 2-4 front to
-//               back; optional fused combined loss.
+//   k_sort_tiles  tile: its keys in (depth, Gaussian index) order.
+//   k_forward   tile: Eqs. 2-4 front to back; optional fused combined loss.
 //   k_backward  tile: reverse compositing; per-record screen-space gradients.
 //   k_bproject  record: chain rule to parameters and pose; per-cell pose partials.
 //   k_finalize  view: FP64 sums of the loss and pose partials; (tracking) the decoupled
@@ -637,6 +637,12 @@ cudaError_t launch_upload_views(const ViewInfo *host_views, int V, ViewInfo *dev
 cudaError_t launch_project(const ProjectLaunch &L, cudaStream_t st);
 cudaError_t launch_scan_tiles(const WsPtrs &ws, const Dims &d, cudaStream_t st);
 cudaError_t launch_emit(const WsPtrs &ws, const Dims &d, cudaStream_t st);
+cudaError_t launch_sort_tiles(const WsPtrs &ws, const Dims &d, cudaStream_t st);
+// Before a forward: every tile's list in depth order, unless the device-wide radix sort
+// (GS_SCHED_RADIX) has already made it.
+inline cudaError_t launch_depth_order(const WsPtrs &ws, const Dims &d, cudaStream_t st) {
+    return d.flags & GS_SCHED_RADIX ? cudaSuccess : launch_sort_tiles(ws, d, st);
+}
 
 struct ForwardLaunch {
     WsPtrs ws;

@@ -1,6 +1,6 @@
 // radix_sort.cu -- the front-to-back order of Eqs. 2-4 as one device-wide LSD radix sort
 // of every (Gaussian, tile) pair on the key (tile, depth), the alternative to the per-tile
-// sort inside the forward (tile_sort.cuh), picked by the launch schedule (GS_SCHED_RADIX).
+// sort (tile_sort.cu), picked by the launch schedule (GS_SCHED_RADIX).
 //
 // k_emit (in this mode) writes each pair as the 64-bit key tile << 32 | bits(depth) (the
 // depth is positive, so its IEEE bits order as unsigned integers) with the record as the

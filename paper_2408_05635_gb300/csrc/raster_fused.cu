@@ -19,7 +19,6 @@
 #include "bwd_walk.cuh"
 #include "fwd_walk.cuh"
 #include "gs_internal.cuh"
-#include "tile_sort.cuh"
 
 namespace gsk {
 
@@ -44,12 +43,6 @@ __device__ __forceinline__ void stage_one(const TrackTileLaunch &L, uint32_t r, 
 
 }  // namespace
 
-// One scratch of shared memory holds the sort's two key buffers, then each warp's
-// transposed rows of the reverse walk.
-constexpr int kFusedWarps = kTilePix / 32;
-constexpr int kFusedRows = kFusedWarps * kWalkFloats<true> * (int)sizeof(float);
-constexpr int kFusedScratch = 2 * kSortSmemKeys * 8 > kFusedRows ? 2 * kSortSmemKeys * 8 : kFusedRows;
-
 // Four blocks per SM (64 registers a thread): with five (48 registers) the walks spill
 // and issue more instructions, and the kernel is slower.
 template <int NB, int LW>
@@ -63,8 +56,7 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
     __shared__ float4 sP1[NB];                     // (kuu, lo, -1/(2 kuu), -1/(2 kvv)): the stride of sP0, sC
     __shared__ __align__(16) uint16_t sList[kTilePix / 32][NB];  // byte offsets: 16 x batch position
     __shared__ float sAcc[NB * A::kStride];
-    __shared__ __align__(16) unsigned char sScratch[kFusedScratch];
-    unsigned long long *sKeys = reinterpret_cast<unsigned long long *>(sScratch);
+    __shared__ __align__(16) float sRows[kTilePix / 32][kWalkFloats<true>];  // the reverse walk's transposed rows
     __shared__ int s_view;
     __shared__ float s_loss[kTilePix / 32];
     __shared__ uint32_t s_nmax;
@@ -94,9 +86,6 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
 
     uint32_t start;
     const uint32_t n = tile_entries(L.ws, L.d, tile, start);
-    // this tile's list in (depth, Gaussian) order, unless the device-wide radix sort
-    // (GS_SCHED_RADIX) has already ordered it
-    if (!(L.d.flags & GS_SCHED_RADIX)) sort_tile(L.ws, start, (int)n, sKeys);
 
     // this pixel's targets: loaded once the first batch is staged (below), so their
     // latency (host memory when the frame is read in place) passes during the forward walk
@@ -198,7 +187,7 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
     for (int off = 16; off > 0; off >>= 1) wlast = max(wlast, __shfl_xor_sync(0xffffffffu, wlast, off));
     if (lane == 0 && wlast) atomicMax(&s_nmax, wlast);
     const PixUp up{g0, g1, g2, gD, gS};
-    float *buf = reinterpret_cast<float *>(sScratch) + warp * kWalkFloats<true>;
+    float *buf = sRows[warp];
     store_planes<true>(buf, up, lane);
     float GB = 0.f;  // g . (colour, depth, 1) of everything behind, back-to-front
     // From the batch the forward staged last down to the first.  The staged one needs no
@@ -281,7 +270,8 @@ cudaError_t launch_track_tile(const TrackTileLaunch &L, cudaStream_t st) {
     const uint32_t nb = L.d.fwd_batch ? L.d.fwd_batch : (uint32_t)kBatch;
     if (nb > tile_threads(L.d) || (L.d.bwd_batch ? L.d.bwd_batch : (uint32_t)kBatch) != nb)
         return cudaErrorInvalidValue;
-    cudaError_t e;
+    cudaError_t e = launch_depth_order(L.ws, L.d, st);
+    if (e != cudaSuccess) return e;
     switch (nb) {
         case 256: e = launch_track_tile_lw<256>(L, st); break;
         case 128: e = launch_track_tile_lw<128>(L, st); break;

@@ -1,8 +1,7 @@
 // raster_fwd.cu -- front-to-back compositing of colour, depth and silhouette.
 //
-// One block per tile (16 x 16 by default), one thread per pixel.  The block first sorts its tile's
-// list (tile_sort.cuh).  For pixel p and the tile's
-// Gaussians in (depth, index) order:
+// One block per tile (16 x 16 by default), one thread per pixel.  For pixel p and the tile's
+// Gaussians in (depth, index) order (tile_sort.cu):
 //   C(p) = sum_i c_i a_i T_i   (Eq. 2)
 //   D(p) = sum_i d_i a_i T_i   (Eq. 3, d_i = camera-frame depth of the mean)
 //   S(p) = sum_i a_i T_i       (Eq. 4)
@@ -22,7 +21,6 @@
 // backward and its value is reduced per tile in double-float (summed per view by k_finalize).
 #include "fwd_walk.cuh"
 #include "gs_internal.cuh"
-#include "tile_sort.cuh"
 
 namespace gsk {
 
@@ -37,7 +35,6 @@ __global__ void __launch_bounds__(kTilePix, 5) k_forward(ForwardLaunch L) {
     __shared__ float4 sP0[NB], sC[NB], sBox[NB];
     __shared__ float4 sP1[NB];                     // (kuu, lo, -1/(2 kuu), -1/(2 kvv)): the stride of sP0, sC
     __shared__ __align__(16) uint16_t sList[kTilePix / 32][NB];  // byte offsets: 16 x batch position
-    __shared__ unsigned long long sKeys[2 * kSortSmemKeys];  // the sort's two buffers
     __shared__ int s_view;
     __shared__ float s_loss[kTilePix / 32];
     __shared__ unsigned long long s_count[2];
@@ -67,9 +64,6 @@ __global__ void __launch_bounds__(kTilePix, 5) k_forward(ForwardLaunch L) {
 
     uint32_t start;
     const uint32_t n = tile_entries(L.ws, L.d, tile, start);
-    // this tile's list in (depth, Gaussian) order, unless the device-wide radix sort
-    // (GS_SCHED_RADIX) has already ordered it
-    if (!(L.d.flags & GS_SCHED_RADIX)) sort_tile(L.ws, start, (int)n, sKeys);
     FwdPixel walk{1.f, 0.f, 0.f, 0.f, 0.f, 0u, 0u, !inside};
     uint32_t n_eval = 0, n_contrib = 0;
     // with the loss: this pixel's targets, loaded once the first batch is staged so their
@@ -215,7 +209,8 @@ cudaError_t launch_forward(const ForwardLaunch &L, cudaStream_t st) {
     // a batch stages at most one Gaussian per thread of the tile block
     const uint32_t nb = L.d.fwd_batch ? L.d.fwd_batch : (uint32_t)kBatch;
     if (nb > tile_threads(L.d)) return cudaErrorInvalidValue;
-    cudaError_t e;
+    cudaError_t e = launch_depth_order(L.ws, L.d, st);
+    if (e != cudaSuccess) return e;
     switch (L.d.fwd_batch) {
         case 0:
         case 256: e = launch_forward_lw<256>(L, st); break;
