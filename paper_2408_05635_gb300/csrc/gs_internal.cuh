@@ -37,8 +37,6 @@ constexpr int kBatch = 256;               // default (and largest) compositing b
 // bytes: NB must not exceed 256 nor the tile's thread count (the host checks the latter).
 static_assert(kBatch <= kTilePix && kBatch <= 256, "a batch stages at most one Gaussian per tile thread");
 constexpr int kSubMax = 4;                // most per-tile sub-buckets a workspace is laid out for
-constexpr int kBigCell = 2;               // large records a cell needs to list them for k_emit's extra blocks
-constexpr int kBigListCap = 2048;         // entries of that list (a listed record per extra warp and pass: 4)
 
 enum ErrFlag : uint32_t { kErrRecords = 1u, kErrPairs = 2u, kErrTimeout = 4u };
 
@@ -68,7 +66,7 @@ struct DevHeader {
     unsigned long long bwd_evals;    // footprints evaluated by k_backward
     unsigned long long bwd_contrib;  // ... of which were differentiated
     uint32_t max_tile;               // longest tile list of the projection
-    uint32_t n_big;                  // records listed in WsPtrs::big (the scan copies the count)
+    uint32_t pad0;
     unsigned long long pad1;
 };
 static_assert(sizeof(DevHeader) == 64, "DevHeader layout");
@@ -124,11 +122,6 @@ struct WsPtrs {
     uint32_t *tile_start;  // T x S + 1, exclusive scan of the counts
     uint32_t *cursor;      // T x S, emission cursors
     uint32_t *tile_order;  // T, tiles by descending list length (launch order of the tile kernels)
-    uint32_t *big;         // kBigListCap: large records of crowded cells (more than kSoloTiles
-                           // candidate tiles, kBigCell of them in one cell), listed by k_project
-                           // (count at tile_cnt[T x S], moved to hdr->n_big by the scan) and
-                           // emitted by k_emit's extra blocks
-    uint8_t *big_listed;   // V x nblk x 256: 1 where the record is in `big` (its cell's warps skip it)
     Rec *rec;              // V x nblk x 256 record slots
     RecGrad *rec_grad;     // same slots
     unsigned long long *keys;  // pair_capacity
@@ -288,47 +281,6 @@ __device__ __forceinline__ void tile_rect(const ViewInfo &vi, float mx, float my
     ty0 = py0 >> vi.tile_lh; ty1 = py1 >> vi.tile_lh;
 }
 
-// Does the support ellipse q(d) = a dx^2 + 2 b dx dy + c dy^2 <= dmax2 meet the
-// rectangle of pixel centres [x0, x1] x [y0, y1]?  The minimum of the convex form over
-// the rectangle is 0 when the centre is inside, otherwise it lies on an edge, where
-// it is a 1-D quadratic minimised in closed form (ia = 1/a, ic = 1/c).  The minimiser
-// only has to be close: the threshold carries a relative margin of 1e-3, far above the
-// FP32 error, so no tile with a pixel at alpha >= alpha_min is dropped.  Every operation
-// is an explicitly rounded intrinsic so k_project and k_emit take identical decisions.
-__device__ __forceinline__ float qform(float a, float b, float c, float dx, float dy) {
-    return __fadd_rn(__fadd_rn(__fmul_rn(a, __fmul_rn(dx, dx)), __fmul_rn(2.f, __fmul_rn(b, __fmul_rn(dx, dy)))),
-                     __fmul_rn(c, __fmul_rn(dy, dy)));
-}
-
-__device__ __forceinline__ bool ellipse_meets_rect(float mx, float my, float a, float b, float c, float ia, float ic,
-                                                   float dmax2, float x0, float x1, float y0, float y1) {
-    if (!(dmax2 < INFINITY)) return true;
-    if (mx >= x0 && mx <= x1 && my >= y0 && my <= y1) return true;
-    const float lx = __fsub_rn(x0, mx), hx = __fsub_rn(x1, mx);
-    const float ly = __fsub_rn(y0, my), hy = __fsub_rn(y1, my);
-    const float nb = -b;
-    float best = INFINITY;
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        const float dx = e ? hx : lx;  // vertical edge: dy free, minimum at dy = -b dx / c
-        const float dy = fminf(fmaxf(__fmul_rn(__fmul_rn(nb, dx), ic), ly), hy);
-        best = fminf(best, qform(a, b, c, dx, dy));
-        const float ey = e ? hy : ly;  // horizontal edge: dx free, minimum at dx = -b dy / a
-        const float ex = fminf(fmaxf(__fmul_rn(__fmul_rn(nb, ey), ia), lx), hx);
-        best = fminf(best, qform(a, b, c, ex, ey));
-    }
-    return best <= __fadd_rn(__fmul_rn(dmax2, 1.001f), 1e-3f);
-}
-
-// Pixel-centre rectangle of tile (tx, ty) >= 0, clipped to the image.
-__device__ __forceinline__ void tile_bounds(const ViewInfo &vi, int tx, int ty, float &x0, float &x1, float &y0,
-                                            float &y1) {
-    x0 = (float)(tx << vi.tile_lw);
-    y0 = (float)(ty << vi.tile_lh);
-    x1 = (float)min(((tx + 1) << vi.tile_lw) - 1, vi.width - 1);
-    y1 = (float)min(((ty + 1) << vi.tile_lh) - 1, vi.height - 1);
-}
-
 // ------------------------------------------------------------------ per-tile footprint
 //
 // For a tile with origin (x0, y0) and tile-local pixel centre (u, v) = (px - x0, py - y0),
@@ -429,19 +381,19 @@ __device__ __forceinline__ float diff_of_products(float a, float b, float c, flo
 }
 
 // Tiles [a0, a1] of row ty (within the record's tile columns [tx0, tx1]) that the support
-// ellipse q(d) <= R, R = dmax2 (1 + 1e-3) + 1e-3 (the margin of ellipse_meets_rect), meets.
+// ellipse q(d) <= R, R = dmax2 (1 + 1e-3) + 1e-3, meets.
 // The ellipse cut by the row's band of pixel centres [y0, y1] is convex, so its x-extent is
 // one interval: on the right boundary x = mx + (-b dy + sqrt(a R - det dy^2)) / a, concave
 // in dy = y - my, the maximum mx + sqrt(R c / det) is reached at dy = -b sqrt(R / (c det)),
 // and outside the band at the nearer band edge; the left boundary mirrors it.  A tile
 // meets the ellipse iff its pixel-centre columns overlap that interval, so this finds the
 // same tiles as testing each tile of the row, at the cost of one row.  The interval is
-// widened by 1e-3 px + 1e-6 |x| against the rounding of the square roots.  Explicitly
-// rounded operations: k_project and k_emit enumerate identical tiles.  The quantities that
+// widened by 1e-3 px + 1e-6 |x| against the rounding of the square roots, and by 4e-7 of
+// the chord's centre -b dy / a (that of a long thin footprint close to the camera is
+// thousands of pixels off, and carries that much rounding).  Explicitly rounded operations: k_project and k_emit enumerate identical tiles.  The quantities that
 // do not depend on the row (RowSpan) are computed once per record by row_span_setup.
 struct RowSpan {
-    float mx, my, b, R, det, Y, X, t, ia, aR;  // aR = a R
-    bool all;                                  // unbounded support: every column
+    float mx, my, b, det, aR, Y, X, t, ia;  // aR = a R, infinite with an unbounded support
 };
 
 __device__ __forceinline__ RowSpan row_span_setup(float mx, float my, float a, float b, float c, float dmax2) {
@@ -449,13 +401,12 @@ __device__ __forceinline__ RowSpan row_span_setup(float mx, float my, float a, f
     s.mx = mx;
     s.my = my;
     s.b = b;
-    s.all = !(dmax2 < INFINITY);
-    s.R = __fadd_rn(__fmul_rn(dmax2, 1.001f), 1e-3f);
+    const float R = __fadd_rn(__fmul_rn(dmax2, 1.001f), 1e-3f);
     s.det = diff_of_products(a, c, b, b);
-    s.aR = __fmul_rn(a, s.R);
+    s.aR = __fmul_rn(a, R);
     s.Y = __fsqrt_rn(__fdiv_rn(s.aR, s.det));                         // y half-extent of the ellipse
-    s.X = __fsqrt_rn(__fdiv_rn(__fmul_rn(s.R, c), s.det));            // x half-extent of the ellipse
-    s.t = __fmul_rn(b, __fsqrt_rn(__fdiv_rn(s.R, __fmul_rn(c, s.det))));  // |dy| of the x-extremes
+    s.X = __fsqrt_rn(__fdiv_rn(__fmul_rn(R, c), s.det));            // x half-extent of the ellipse
+    s.t = __fmul_rn(b, __fsqrt_rn(__fdiv_rn(R, __fmul_rn(c, s.det))));  // |dy| of the x-extremes
     s.ia = __fdiv_rn(1.f, a);
     return s;
 }
@@ -464,7 +415,7 @@ __device__ __forceinline__ void row_span(const ViewInfo &vi, const RowSpan &s, i
                                          int &a1) {
     a0 = tx0;
     a1 = tx1;
-    if (s.all) return;
+    if (!(s.aR < INFINITY)) return;  // every column
     const float yb0 = (float)(ty << vi.tile_lh), yb1 = (float)min(((ty + 1) << vi.tile_lh) - 1, vi.height - 1);
     const float ly = fmaxf(__fsub_rn(yb0, s.my), -s.Y), hy = fminf(__fsub_rn(yb1, s.my), s.Y);
     if (!(ly <= hy)) {
@@ -485,8 +436,9 @@ __device__ __forceinline__ void row_span(const ViewInfo &vi, const RowSpan &s, i
         xl = -s.X;
     else
         xl = fminf(__fsub_rn(cl, __fmul_rn(rl, s.ia)), __fsub_rn(ch, __fmul_rn(rh, s.ia)));
-    xl = __fsub_rn(__fadd_rn(s.mx, xl), __fadd_rn(1e-3f, __fmul_rn(1e-6f, fabsf(__fadd_rn(s.mx, xl)))));
-    xr = __fadd_rn(__fadd_rn(s.mx, xr), __fadd_rn(1e-3f, __fmul_rn(1e-6f, fabsf(__fadd_rn(s.mx, xr)))));
+    const float w = __fadd_rn(1e-3f, __fmul_rn(4e-7f, fmaxf(fabsf(cl), fabsf(ch))));
+    xl = __fsub_rn(__fadd_rn(s.mx, xl), __fadd_rn(w, __fmul_rn(1e-6f, fabsf(__fadd_rn(s.mx, xl)))));
+    xr = __fadd_rn(__fadd_rn(s.mx, xr), __fadd_rn(w, __fmul_rn(1e-6f, fabsf(__fadd_rn(s.mx, xr)))));
     // tile tx spans pixel centres [TW tx, TW tx + TW - 1]: it meets [xl, xr] iff
     // TW tx + TW - 1 >= xl and TW tx <= xr (TW a power of two: multiplying by 1 / TW is
     // exact, the same as dividing)

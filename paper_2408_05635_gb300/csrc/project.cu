@@ -30,55 +30,133 @@ __device__ __forceinline__ bool record_rect(const ViewInfo &vi, float4 A, float4
     return tx0 <= tx1 && ty0 <= ty1;
 }
 
-__device__ __forceinline__ bool tile_hit(const ViewInfo &vi, float4 A, float4 B, float ia, float ic, int tx, int ty) {
-    float x0, x1, y0, y1;
-    tile_bounds(vi, tx, ty, x0, x1, y0, y1);
-    return ellipse_meets_rect(A.x, A.y, B.x, B.y, B.z, ia, ic, B.w, x0, x1, y0, y1);
+// The tiles of a block's records (k_project counts them, k_emit writes a key into each).
+// Work is handed out by tile rows: the rows of all the block's rectangles are numbered
+// through, each thread takes every kBlock-th and walks the row's span of tiles, so a
+// Gaussian close to the camera, whose rectangle spans thousands of tiles, and a warp of
+// uneven ones are spread over the block.  The tiles are gathered in shared counters over the
+// block's own tile box first (neighbouring Gaussians share their tiles: a map along a
+// Morton curve or built frame by frame), which leaves one global atomic per tile and block
+// instead of one per (record, tile) pair.  Both kernels run this code on the same floats, so
+// they enumerate the same tiles.
+//
+// Before, a lane walked its own record and a warp or extra blocks the large ones, with an
+// atomic per pair: what bound both kernels was the atomics' rate and round trips.  8 views
+// of 1M Gaussians (29 pairs a record): k_project 185 -> 113 us, k_emit 161 -> 74; one view
+// of 1M at 1200 x 680 (10 pairs): 48 -> 29 and 64 -> 38; 2M in FP16 (4.6): 80 -> 63 and 87
+// -> 40 (k_emit's times hold its wait for the scan).  Unchanged within a microsecond where
+// latency counts (200k, 37k records) and on footprints a pixel wide (1.8 pairs a record: 57
+// -> 61 and 61 -> 55 us).
+constexpr int kSoloRows = 4;     // records of no more rows: handing their rows out costs more than walking them
+                                 // (1.8 pairs a record: a window of 864 us took 887)
+constexpr int kBoxTiles = 3328;  // a 1200 x 680 image has 3,225 tiles; beyond, atomics go to global memory
+
+struct RowRec {  // one record's rows
+    float4 a;    // mu'_x, mu'_y, b, det
+    float4 b;    // aR, Y, X, t
+    float ia;
+    int tx0, tx1, ty0;
+};
+
+struct BinSmem {
+    RowRec rec[kBlock];
+    uint32_t pre[kBlock + 1];  // rows before each record
+    uint32_t box[kBoxTiles];
+    int4 warp_box[kWarps];     // first tile column and row, last column and row
+    uint2 warp_rows[kWarps];   // rows, and the most of one record
+};
+
+// Posts the warp's rows and tile box (block_box reads them after a barrier); returns the rows
+// of the warp's lanes before this one.
+__device__ __forceinline__ uint32_t post_rows(BinSmem &sm, bool has, int tx0, int tx1, int ty0, int ty1) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t rows = has ? (uint32_t)(ty1 - ty0 + 1) : 0u;
+    uint32_t incl = rows;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += v;
+    }
+    const int lx = __reduce_min_sync(0xffffffffu, has ? tx0 : 0x7fffffff), hx = __reduce_max_sync(0xffffffffu, has ? tx1 : -1);
+    const int ly = __reduce_min_sync(0xffffffffu, has ? ty0 : 0x7fffffff), hy = __reduce_max_sync(0xffffffffu, has ? ty1 : -1);
+    const uint32_t most = __reduce_max_sync(0xffffffffu, rows);
+    if (lane == 31) {
+        sm.warp_box[warp] = make_int4(lx, ly, hx, hy);
+        sm.warp_rows[warp] = make_uint2(incl, most);
+    }
+    return incl - rows;
 }
 
-// Tiles met by each lane's own record (mine = the lane has one).  A lane whose tile
-// rectangle has at most kSoloTiles candidates tests them alone; larger rectangles (a
-// Gaussian close to the camera can span thousands of tiles) are split over the 32 lanes
-// of the warp, so one of them never holds the rest of the grid.  body(src lane, tile,
-// record's A, record's tag) runs once for every tile the support meets.
-constexpr int kSoloTiles = 24;
+struct BlockBox {
+    int x, y, w, area;      // first tile, columns, tiles (0: gathered in global memory)
+    bool boxed, solo;
+    uint32_t before, rows;  // rows of the warps before this one, of the block
+};
 
-template <bool SOLO = true, class Body>
-__device__ __forceinline__ void record_tiles(bool mine, const ViewInfo &vi, float4 A, float4 B, uint32_t tag, int lane,
-                                             Body &&body) {
-    int tx0 = 1, tx1 = 0, ty0 = 1, ty1 = 0;
-    const bool has = mine && record_rect(vi, A, B, tx0, tx1, ty0, ty1);
-    const int rw = tx1 - tx0 + 1;
-    const int count = has ? rw * (ty1 - ty0 + 1) : 0;
-    if (SOLO && has && count <= kSoloTiles) {
-        const RowSpan span = row_span_setup(A.x, A.y, B.x, B.y, B.z, B.w);
-        for (int ty = ty0; ty <= ty1; ++ty) {
-            int a0, a1;
-            row_span(vi, span, ty, tx0, tx1, a0, a1);
-            for (int tx = a0; tx <= a1; ++tx) body(lane, vi.tile_base + (uint32_t)(ty * vi.tiles_x + tx), A, tag);
-        }
+__device__ __forceinline__ BlockBox block_box(const BinSmem &sm) {
+    const int warp = threadIdx.x >> 5;
+    int4 q = sm.warp_box[0];
+    uint2 r = sm.warp_rows[0];
+    BlockBox o;
+    o.before = warp > 0 ? r.x : 0u;
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) {
+        const int4 p = sm.warp_box[w];
+        const uint2 c = sm.warp_rows[w];
+        q = make_int4(min(q.x, p.x), min(q.y, p.y), max(q.z, p.z), max(q.w, p.w));
+        o.before += w < warp ? c.x : 0u;
+        r = make_uint2(r.x + c.x, max(r.y, c.y));
     }
-    uint32_t big = __ballot_sync(0xffffffffu, count > kSoloTiles);
-    while (big) {
-        const int src = __ffs(big) - 1;
-        big &= big - 1;
-        float4 As, Bs;
-        As.x = __shfl_sync(0xffffffffu, A.x, src);
-        As.y = __shfl_sync(0xffffffffu, A.y, src);
-        As.z = __shfl_sync(0xffffffffu, A.z, src);
-        As.w = __shfl_sync(0xffffffffu, A.w, src);
-        Bs.x = __shfl_sync(0xffffffffu, B.x, src);
-        Bs.y = __shfl_sync(0xffffffffu, B.y, src);
-        Bs.z = __shfl_sync(0xffffffffu, B.z, src);
-        Bs.w = __shfl_sync(0xffffffffu, B.w, src);
-        const uint32_t tg = __shfl_sync(0xffffffffu, tag, src);
-        const int sx0 = __shfl_sync(0xffffffffu, tx0, src), sy0 = __shfl_sync(0xffffffffu, ty0, src);
-        const int srw = __shfl_sync(0xffffffffu, rw, src), scount = __shfl_sync(0xffffffffu, count, src);
-        const float ia = __fdividef(1.f, Bs.x), ic = __fdividef(1.f, Bs.z);
-        for (int t = lane; t < scount; t += 32) {
-            const int ty = sy0 + t / srw, tx = sx0 + t % srw;
-            if (tile_hit(vi, As, Bs, ia, ic, tx, ty)) body(src, vi.tile_base + (uint32_t)(ty * vi.tiles_x + tx), As, tg);
+    o.rows = r.x;
+    o.solo = r.y <= (uint32_t)kSoloRows;
+    o.x = q.x;
+    o.y = q.y;
+    o.w = q.z - q.x + 1;
+    o.boxed = r.x > 0u && (int64_t)o.w * (q.w - q.y + 1) <= kBoxTiles;
+    o.area = o.boxed ? o.w * (q.w - q.y + 1) : 0;
+    return o;
+}
+
+__device__ __forceinline__ void put_rows(RowRec &r, float4 A, float4 B, int tx0, int tx1, int ty0) {
+    const RowSpan s = row_span_setup(A.x, A.y, B.x, B.y, B.z, B.w);
+    r.a = make_float4(s.mx, s.my, s.b, s.det);
+    r.b = make_float4(s.aR, s.Y, s.X, s.t);
+    r.ia = s.ia;
+    r.tx0 = tx0;
+    r.tx1 = tx1;
+    r.ty0 = ty0;
+}
+
+// body(tile row, first tile column, last) for the rows of this thread's own record.
+template <class Body>
+__device__ __forceinline__ void for_own_rows(const ViewInfo &vi, float4 A, float4 B, int tx0, int tx1, int ty0, int ty1,
+                                             Body &&body) {
+    const RowSpan s = row_span_setup(A.x, A.y, B.x, B.y, B.z, B.w);
+    for (int ty = ty0; ty <= ty1; ++ty) {
+        int a0, a1;
+        row_span(vi, s, ty, tx0, tx1, a0, a1);
+        if (a0 <= a1) body(ty, a0, a1);
+    }
+}
+
+// body(record, tile row, first tile column, last) for this thread's share of the rows of
+// nrec > 0 records.
+template <class Body>
+__device__ __forceinline__ void for_rows(const BinSmem &sm, int nrec, const ViewInfo &vi, Body &&body) {
+    const uint32_t rows = sm.pre[nrec];
+    for (uint32_t f = threadIdx.x; f < rows; f += kBlock) {
+        int lo = 0, hi = nrec - 1;  // the last record whose prefix is at most f
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (sm.pre[mid] <= f) lo = mid; else hi = mid - 1;
         }
+        const RowRec &r = sm.rec[lo];
+        const int ty = r.ty0 + (int)(f - sm.pre[lo]);
+        const float4 ra = r.a, rb = r.b;
+        const RowSpan s{ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w, r.ia};
+        int a0, a1;
+        row_span(vi, s, ty, r.tx0, r.tx1, a0, a1);
+        if (a0 <= a1) body(lo, ty, a0, a1);
     }
 }
 
@@ -238,8 +316,6 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(WsPtrs ws, Dims d) 
     }
     if (tid == 0) {
         ws.tile_start[TS] = (uint32_t)min(carry, (unsigned long long)0xffffffffu);
-        ws.hdr->n_big = ws.tile_cnt[TS];  // the large records k_project listed, zeroed for the next pass
-        ws.tile_cnt[TS] = 0u;
     }
     __syncthreads();
     {  // exclusive scan of the buckets, one bucket per thread
@@ -428,8 +504,6 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_top(WsPtrs ws, Dims d) {
     __syncthreads();
     if (tid == 0) {
         ws.tile_start[TS] = (uint32_t)min(total, (unsigned long long)0xffffffffu);
-        ws.hdr->n_big = ws.tile_cnt[TS];  // the large records k_project listed, zeroed for the next pass
-        ws.tile_cnt[TS] = 0u;
         ws.hdr->max_tile = s_max;
         ws.hdr->n_rec = s_rec;
         ws.hdr->n_pairs = total;
@@ -503,12 +577,6 @@ cudaError_t launch_scan_tiles(const WsPtrs &ws, const Dims &d, cudaStream_t st) 
     return e;
 }
 
-// A block's large records (more than kSoloTiles candidate tiles) are counted by all its
-// threads at once, each taking (record, tile) pairs of their concatenated rectangles,
-// instead of one record after the other by the warp that holds it; kBigPerBlock of them,
-// a further one by its warp.
-constexpr int kBigPerBlock = 64;
-
 template <int DT, bool ISO>
 __global__ void __launch_bounds__(kBlock, 6) k_project(ProjectLaunch L) {
     griddep_wait();  // the predecessor's results are visible from here on
@@ -518,14 +586,11 @@ __global__ void __launch_bounds__(kBlock, 6) k_project(ProjectLaunch L) {
     __shared__ float sRt[12];
     __shared__ ViewInfo sv;
     __shared__ uint32_t warp_off[kWarps];
-    __shared__ float4 sbA[kBigPerBlock], sbB[kBigPerBlock];
-    __shared__ int4 sbR[kBigPerBlock];         // first tile column and row, columns, candidates
-    __shared__ uint32_t sbPre[kBigPerBlock + 1], sbSub[kBigPerBlock], s_nbig;
+    __shared__ BinSmem sm;
     const uint32_t cell = (uint32_t)v * (uint32_t)L.d.nblk + (uint32_t)b;
     if (tid == 0) {
         load_pose(L.poses + 7 * v, sRt);
         sv = L.ws.views[v];
-        s_nbig = 0u;
     }
     __syncthreads();
     if (b == 0 && tid < 12) L.ws.view_rt[12 * v + tid] = sRt[tid];
@@ -536,8 +601,8 @@ __global__ void __launch_bounds__(kBlock, 6) k_project(ProjectLaunch L) {
     const int64_t i = (int64_t)b * kBlock + tid;
     const Settings &S = L.s;
     float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = A, C = A;
-    bool vis = false, big = false;
-    int4 rect = make_int4(0, 0, 0, 0);
+    bool vis = false;
+    int tx0 = 0, tx1 = 0, ty0 = 0, ty1 = 0;
     if (i < L.d.n) {
         const float mx = __ldg(L.g.means + 3 * i), my = __ldg(L.g.means + 3 * i + 1), mz = __ldg(L.g.means + 3 * i + 2);
         const float x = cam_coord(sRt, 0, mx, my, mz);
@@ -631,10 +696,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_project(ProjectLaunch L) {
                     C = make_float4(ld_attr<DT>(L.g.rgb, 3 * i), ld_attr<DT>(L.g.rgb, 3 * i + 1),
                                     ld_attr<DT>(L.g.rgb, 3 * i + 2),
                                     __uint_as_float((uint32_t)((int64_t)v * L.d.n + i)));
-                    int tx0, tx1, ty0, ty1;
                     vis = record_rect(vi, A, B, tx0, tx1, ty0, ty1);
-                    big = vis && (tx1 - tx0 + 1) * (ty1 - ty0 + 1) > kSoloTiles;
-                    rect = make_int4(tx0, ty0, tx1 - tx0 + 1, (tx1 - tx0 + 1) * (ty1 - ty0 + 1));
                 }
             }
         }
@@ -642,90 +704,55 @@ __global__ void __launch_bounds__(kBlock, 6) k_project(ProjectLaunch L) {
     // compaction into this block's cell: visible Gaussians take the first slots, in order
     const uint32_t ballot = __ballot_sync(0xffffffffu, vis);
     if (lane == 0) warp_off[warp] = __popc(ballot);
+    const uint32_t before = post_rows(sm, vis, tx0, tx1, ty0, ty1);
     __syncthreads();
-    if (tid == 0) {
-        uint32_t run = 0;
-        for (int w = 0; w < kWarps; ++w) {
-            const uint32_t c = warp_off[w];
-            warp_off[w] = run;
-            run += c;
-        }
-        L.ws.cell_cnt[cell] = run;
+    uint32_t nrec = 0, slot = __popc(ballot & ((1u << lane) - 1u));
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        const uint32_t c = warp_off[w];
+        slot += w < warp ? c : 0u;
+        nrec += c;
     }
-    // the block's large records, for the block-wide count below
-    const uint32_t nsub = L.d.S;
-    bool mine_solo = vis;
-    if (big) {
-        const uint32_t k = atomicAdd(&s_nbig, 1u);
-        if (k < (uint32_t)kBigPerBlock) {
-            sbA[k] = A;
-            sbB[k] = B;
-            sbR[k] = rect;
-            sbSub[k] = (uint32_t)i & (nsub - 1);
-            mine_solo = false;
-        }
-    }
-    __syncthreads();
+    if (tid == 0) L.ws.cell_cnt[cell] = nrec;
+    if (nrec == 0) return;
+    const BlockBox q = block_box(sm);
+    for (int k = tid; k < q.area; k += kBlock) sm.box[k] = 0u;
     if (vis) {
-        const uint32_t rec = cell * kCell + warp_off[warp] + __popc(ballot & ((1u << lane) - 1u));
+        const uint32_t rec = cell * kCell + slot;
         Rec r;
         r.a = A; r.b = B; r.c = C;
         L.ws.rec[rec] = r;
         RecGrad z;
         z.g0 = z.g1 = z.g2 = make_float4(0.f, 0.f, 0.f, 0.f);
         L.ws.rec_grad[rec] = z;
-        // the large records of a cell that holds kBigCell or more: listed for k_emit's extra
-        // blocks while the list has room (the cell's warps emit the others)
-        uint8_t listed = 0;
-        if (big && s_nbig >= (uint32_t)kBigCell) {
-            const uint32_t k = atomicAdd(L.ws.tile_cnt + L.d.T * L.d.S, 1u);
-            if (k < (uint32_t)kBigListCap) {
-                L.ws.big[k] = rec;
-                listed = 1;
-            }
-        }
-        L.ws.big_listed[rec] = listed;
-    }
-    // per-(tile, sub-bucket) pair counts: the block's listed large records by all threads,
-    // every other visible record by its own lane (or, above kSoloTiles, its warp)
-    uint32_t *cnt = L.ws.tile_cnt;
-    const uint32_t nbig = min(s_nbig, (uint32_t)kBigPerBlock);  // block-uniform
-    if (nbig) {
-        if (warp == 0) {  // exclusive prefix of the rectangles' candidate counts
-            uint32_t run = 0;
-            for (uint32_t base = 0; base < nbig; base += 32) {
-                const uint32_t e = base + (uint32_t)lane;
-                const uint32_t c = e < nbig ? (uint32_t)sbR[e].w : 0u;
-                uint32_t incl = c;
-#pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
-                    if (lane >= off) incl += y;
-                }
-                if (e < nbig) sbPre[e] = run + incl - c;
-                run += __shfl_sync(0xffffffffu, incl, 31);
-            }
-            if (lane == 0) sbPre[nbig] = run;
-        }
-        __syncthreads();
-        const uint32_t total = sbPre[nbig];
-        for (uint32_t f = (uint32_t)tid; f < total; f += kBlock) {
-            int lo = 0, hi = (int)nbig - 1;  // the last entry whose prefix is at most f
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (sbPre[mid] <= f) lo = mid; else hi = mid - 1;
-            }
-            const int4 R = sbR[lo];
-            const int t = (int)(f - sbPre[lo]);
-            const int ty = R.y + t / R.z, tx = R.x + t % R.z;
-            const float4 Ab = sbA[lo], Bb = sbB[lo];
-            if (tile_hit(vi, Ab, Bb, __fdividef(1.f, Bb.x), __fdividef(1.f, Bb.z), tx, ty))
-                red_add(cnt + (vi.tile_base + (uint32_t)(ty * vi.tiles_x + tx)) * nsub + sbSub[lo], 1u);
+        if (!q.solo) {
+            put_rows(sm.rec[slot], A, B, tx0, tx1, ty0);
+            sm.pre[slot] = q.before + before;
         }
     }
-    record_tiles(mine_solo, vi, A, B, (uint32_t)i & (nsub - 1), lane, [&](int, uint32_t tile, float4, uint32_t sub) {
-        red_add(cnt + tile * nsub + sub, 1u);
-    });
+    if (tid == 0) sm.pre[nrec] = q.rows;
+    __syncthreads();
+    // pair counts per (tile, sub-bucket of the cell)
+    uint32_t *cnt = L.ws.tile_cnt + vi.tile_base * L.d.S + ((uint32_t)b & (L.d.S - 1));
+    const auto count = [&](int ty, int a0, int a1) {
+        if (q.boxed) {
+            uint32_t *row = sm.box + (ty - q.y) * q.w - q.x;
+            for (int tx = a0; tx <= a1; ++tx) atomicAdd(row + tx, 1u);
+        } else {
+            for (int tx = a0; tx <= a1; ++tx) red_add(cnt + (uint32_t)(ty * vi.tiles_x + tx) * L.d.S, 1u);
+        }
+    };
+    if (q.solo) {
+        if (vis) for_own_rows(vi, A, B, tx0, tx1, ty0, ty1, count);
+    } else {
+        for_rows(sm, (int)nrec, vi, [&](int, int ty, int a0, int a1) { count(ty, a0, a1); });
+    }
+    if (!q.boxed) return;
+    __syncthreads();
+    for (int k = tid; k < q.area; k += kBlock) {
+        const uint32_t c = sm.box[k];
+        if (c) red_add(cnt + (uint32_t)((q.y + k / q.w) * vi.tiles_x + q.x + k % q.w) * L.d.S, c);
+    }
 }
 
 cudaError_t launch_project(const ProjectLaunch &L, cudaStream_t st) {
@@ -763,139 +790,139 @@ __device__ __forceinline__ void put_pair(const WsPtrs &ws, bool radix, uint32_t 
     }
 }
 
-// The emission runs kEmitThreads threads per block, kCell / kEmitThreads blocks per cell,
-// compiled for kEmitMinBlocks resident blocks per SM (64 registers a thread).
-constexpr int kEmitThreads = 64;
-constexpr int kEmitMinBlocks = 16;
-static_assert(kCell % kEmitThreads == 0 && kEmitThreads % 32 == 0, "emission blocks split cells into warps");
-
 // One key per (record, tile met): depth bits (positive floats sort as unsigned ints) in
 // the high word, the record in the low word, stored at the next free slot of the tile's
-// sub-bucket.  One block per cell, one thread per record (record_tiles).
-// Blocks of k_emit after the cells' blocks: each warp emits the pairs of the large records
-// k_project listed (those of cells crowded with them, ws.big), a record at a time with one
-// tile of its rectangle per lane, so the records close to the camera are spread over many
-// warps instead of lengthening the few warps of the cells that hold them.
-constexpr int kBigBlocks = 256;
-
-__device__ __forceinline__ void emit_big(const WsPtrs &ws, const Dims &d, uint32_t gwarp, int lane) {
-    const uint32_t nbig = min(ws.hdr->n_big, (uint32_t)kBigListCap);
-    const uint32_t slots = rec_slots(d);
-    const bool radix = (d.flags & GS_SCHED_RADIX) != 0;
-    for (uint32_t k = gwarp; k < nbig; k += (uint32_t)kBigBlocks * (kEmitThreads / 32)) {
-        const uint32_t r = ws.big[k];
-        if (r >= slots) continue;  // never written past the records (one entry per record)
-        const Rec rec = ws.rec[r];
-        const ViewInfo vi = ws.views[r / ((uint32_t)d.nblk * (uint32_t)kCell)];
-        const uint32_t sub = (uint32_t)((uint64_t)__float_as_uint(rec.c.w) % (uint64_t)d.n) & (d.S - 1);
-        int tx0, tx1, ty0, ty1;
-        if (!record_rect(vi, rec.a, rec.b, tx0, tx1, ty0, ty1)) continue;
-        const int rw = tx1 - tx0 + 1, count = rw * (ty1 - ty0 + 1);
-        const float ia = __fdividef(1.f, rec.b.x), ic = __fdividef(1.f, rec.b.z);
-        for (int t = lane; t < count; t += 32) {
-            const int ty = ty0 + t / rw, tx = tx0 + t % rw;
-            if (!tile_hit(vi, rec.a, rec.b, ia, ic, tx, ty)) continue;
-            const uint32_t tile = vi.tile_base + (uint32_t)(ty * vi.tiles_x + tx);
-            const uint32_t bucket = tile * d.S + sub;
-            const uint32_t slot = atomicAdd(ws.cursor + bucket, 1u);
-            if (slot < ws.tile_start[bucket + 1] && slot < d.pair_cap)
-                put_pair(ws, radix, slot, tile, __float_as_uint(rec.a.z), r);
-            else
-                atomicOr(ws.err, (uint32_t)kErrPairs);
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kEmitThreads, kEmitMinBlocks) k_emit(WsPtrs ws, Dims d) {
+// sub-bucket.  One block per cell: the block counts its pairs per tile as k_project did,
+// reserves each tile's slots with one atomic, and hands them out from shared memory.
+__global__ void __launch_bounds__(kBlock, 6) k_emit(WsPtrs ws, Dims d) {
     // No early griddep_launch_dependents here: the sort's blocks would then be placed while
     // the emission still runs, on whichever SMs free first, and take slots from its own
     // blocks (12 views / 500k Gaussians: a call 2,900 -> 2,969 us; one view of 2M: 1,632 ->
     // 1,709 us).
     griddep_wait();  // the predecessor's results are visible from here on
-    const uint32_t cell_blocks = (uint32_t)d.V * (uint32_t)d.nblk * (uint32_t)(kCell / kEmitThreads);
-    if (blockIdx.x >= cell_blocks) {
-        emit_big(ws, d, (blockIdx.x - cell_blocks) * (kEmitThreads / 32) + (threadIdx.x >> 5), threadIdx.x & 31);
-        return;
-    }
-    // kCell / kEmitThreads blocks per cell, each taking a quarter of the cell's slots: a
-    // cell full of visible Gaussians (neighbours in a map built frame by frame) is spread
-    // over several SMs instead of running as one long block, and empty quarters leave at once
-    const uint32_t cell = blockIdx.x / (uint32_t)(kCell / kEmitThreads);
-    const uint32_t first = (blockIdx.x % (uint32_t)(kCell / kEmitThreads)) * (uint32_t)kEmitThreads;
-    const uint32_t cnt = ws.cell_cnt[cell];
-    const uint32_t slot_id = first + threadIdx.x;  // the record slot of this thread in the cell
-    if ((slot_id & ~31u) >= cnt) return;  // whole warps without records leave
-    const int lane = threadIdx.x & 31;
+    const uint32_t cell = blockIdx.x;
+    const int nrec = (int)ws.cell_cnt[cell];
+    if (nrec == 0) return;
+    __shared__ BinSmem sm;
+    __shared__ uint32_t s_depth[kBlock];
+    const int tid = threadIdx.x;
     const int view = (int)(cell / (uint32_t)d.nblk);
     const ViewInfo vi = ws.views[view];
-    const uint32_t r = cell * kCell + slot_id;
-    const bool mine = slot_id < cnt;
     float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = A;
-    uint32_t sub = 0;
-    if (mine) {
-        const Rec rec = ws.rec[r];
+    int tx0 = 0, tx1 = 0, ty0 = 0, ty1 = 0;
+    bool has = false;
+    if (tid < nrec) {
+        const Rec &rec = ws.rec[cell * kCell + tid];
         A = rec.a;
         B = rec.b;
-        sub = (uint32_t)((uint64_t)__float_as_uint(rec.c.w) % (uint64_t)d.n) & (d.S - 1);
+        has = record_rect(vi, A, B, tx0, tx1, ty0, ty1);
     }
+    const uint32_t before = post_rows(sm, has, tx0, tx1, ty0, ty1);
+    __syncthreads();
+    const BlockBox q = block_box(sm);
+    for (int k = tid; k < q.area; k += kBlock) sm.box[k] = 0u;
+    if (!q.solo && tid < nrec) {
+        put_rows(sm.rec[tid], A, B, tx0, tx1, ty0);
+        sm.pre[tid] = q.before + before;
+        s_depth[tid] = __float_as_uint(A.z);
+    }
+    if (tid == 0) sm.pre[nrec] = q.rows;
+    __syncthreads();
     const bool radix = (d.flags & GS_SCHED_RADIX) != 0;
-    // small rectangles: this lane alone, slot atomics issued eight at a time before the
-    // dependent stores, so a record waits for about one atomic round trip per eight tiles
-    int tx0 = 1, tx1 = 0, ty0 = 1, ty1 = 0;
-    const bool has = mine && record_rect(vi, A, B, tx0, tx1, ty0, ty1);
-    const int rw = tx1 - tx0 + 1;
-    const int count = has ? rw * (ty1 - ty0 + 1) : 0;
-    if (has && count <= kSoloTiles) {
-        uint32_t hits = 0;  // bit (ty - ty0) rw + (tx - tx0) for every tile met
-        const RowSpan span = row_span_setup(A.x, A.y, B.x, B.y, B.z, B.w);
-        for (int ty = ty0; ty <= ty1; ++ty) {
-            int a0, a1;
-            row_span(vi, span, ty, tx0, tx1, a0, a1);
-            if (a0 <= a1) hits |= ((1u << (a1 - a0 + 1)) - 1u) << ((ty - ty0) * rw + (a0 - tx0));
-        }
-        while (hits) {
-            uint32_t bucket[8], slot[8];
-            bool live[8];
+    const uint32_t sub = (cell % (uint32_t)d.nblk) & (d.S - 1), first = cell * kCell;
+    const auto bucket_of = [&](int ty, int tx) { return (vi.tile_base + (uint32_t)(ty * vi.tiles_x + tx)) * d.S + sub; };
+    if (!q.boxed) {
+        const auto emit = [&](uint32_t depth, uint32_t r, int ty, int a0, int a1) {
+            for (int t0 = a0; t0 <= a1; t0 += 4) {  // four atomics in flight before the stores
+                uint32_t slot[4];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                live[k] = hits != 0;
-                const int t = live[k] ? __ffs(hits) - 1 : 0;
-                hits &= hits - 1;
-                bucket[k] = (vi.tile_base + (uint32_t)((ty0 + t / rw) * vi.tiles_x + tx0 + t % rw)) * d.S + sub;
+                for (int k = 0; k < 4; ++k)
+                    if (t0 + k <= a1) slot[k] = atomicAdd(ws.cursor + bucket_of(ty, t0 + k), 1u);
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (t0 + k <= a1) {
+                        const uint32_t bucket = bucket_of(ty, t0 + k);
+                        if (slot[k] < ws.tile_start[bucket + 1] && slot[k] < d.pair_cap)
+                            put_pair(ws, radix, slot[k], bucket / d.S, depth, first + r);
+                        else
+                            atomicOr(ws.err, (uint32_t)kErrPairs);
+                    }
             }
+        };
+        if (!q.solo) {
+            for_rows(sm, nrec, vi, [&](int r, int ty, int a0, int a1) { emit(s_depth[r], (uint32_t)r, ty, a0, a1); });
+        } else if (has) {
+            for_own_rows(vi, A, B, tx0, tx1, ty0, ty1,
+                         [&](int ty, int a0, int a1) { emit(__float_as_uint(A.z), (uint32_t)tid, ty, a0, a1); });
+        }
+        return;
+    }
+    const auto count = [&](int ty, int a0, int a1) {
+        uint32_t *row = sm.box + (ty - q.y) * q.w - q.x;
+        for (int tx = a0; tx <= a1; ++tx) atomicAdd(row + tx, 1u);
+    };
+    uint32_t span[kSoloRows];  // solo: the row's tiles in the box (first | last << 16; empty: 1 | 0)
+    if (q.solo) {
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (live[k]) slot[k] = atomicAdd(ws.cursor + bucket[k], 1u);
+        for (int k = 0; k < kSoloRows; ++k) span[k] = 1u;
+        if (has) {
+            const RowSpan s = row_span_setup(A.x, A.y, B.x, B.y, B.z, B.w);
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (live[k]) {
-                    if (slot[k] < ws.tile_start[bucket[k] + 1] && slot[k] < d.pair_cap)
-                        put_pair(ws, radix, slot[k], bucket[k] / d.S, __float_as_uint(A.z), r);
-                    else
-                        atomicOr(ws.err, (uint32_t)kErrPairs);
+            for (int k = 0; k < kSoloRows; ++k)
+                if (ty0 + k <= ty1) {
+                    int a0, a1;
+                    row_span(vi, s, ty0 + k, tx0, tx1, a0, a1);
+                    if (a0 <= a1) {
+                        span[k] = (uint32_t)(a0 - q.x) | (uint32_t)(a1 - q.x) << 16;
+                        count(ty0 + k, a0, a1);
+                    }
                 }
         }
+    } else {
+        for_rows(sm, nrec, vi, [&](int, int ty, int a0, int a1) { count(ty, a0, a1); });
     }
-    // large rectangles: those k_project listed are emitted by the blocks after the cells'
-    // (emit_big); the warp splits the others
-    const uint32_t rbase = cell * kCell + (slot_id & ~31u);
-    record_tiles<false>(mine && !ws.big_listed[r], vi, A, B, sub, lane,
-                        [&](int src, uint32_t tile, float4 As, uint32_t sb) {
-        const uint32_t bucket = tile * d.S + sb;
-        const uint32_t slot = atomicAdd(ws.cursor + bucket, 1u);
-        if (slot < ws.tile_start[bucket + 1] && slot < d.pair_cap)
-            put_pair(ws, radix, slot, tile, __float_as_uint(As.z), rbase + (uint32_t)src);
-        else
-            atomicOr(ws.err, (uint32_t)kErrPairs);
-    });
+    __syncthreads();
+    for (int k0 = tid; k0 < q.area; k0 += 4 * kBlock) {  // counts to first slots, four tiles in flight
+        uint32_t c[4], at[4], end[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = k0 + k * kBlock;
+            c[k] = i < q.area ? sm.box[i] : 0u;
+            if (c[k]) {
+                const uint32_t bucket = bucket_of(q.y + i / q.w, q.x + i % q.w);
+                at[k] = atomicAdd(ws.cursor + bucket, c[k]);
+                end[k] = ws.tile_start[bucket + 1];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (c[k]) {
+                sm.box[k0 + k * kBlock] = at[k];
+                if (at[k] + c[k] > end[k] || at[k] + c[k] > d.pair_cap) atomicOr(ws.err, (uint32_t)kErrPairs);
+                if (at[k] + c[k] > end[k]) sm.box[k0 + k * kBlock] = d.pair_cap;  // never past the tile's slots
+            }
+    }
+    __syncthreads();
+    const auto put = [&](uint32_t depth, uint32_t r, int ty, int a0, int a1) {
+        uint32_t *row = sm.box + (ty - q.y) * q.w - q.x;
+        for (int tx = a0; tx <= a1; ++tx) {
+            const uint32_t slot = atomicAdd(row + tx, 1u);
+            if (slot < d.pair_cap)
+                put_pair(ws, radix, slot, vi.tile_base + (uint32_t)(ty * vi.tiles_x + tx), depth, first + r);
+        }
+    };
+    if (q.solo) {
+#pragma unroll
+        for (int k = 0; k < kSoloRows; ++k)
+            put(__float_as_uint(A.z), (uint32_t)tid, ty0 + k, q.x + (int)(span[k] & 0xffffu), q.x + (int)(span[k] >> 16));
+    } else {
+        for_rows(sm, nrec, vi, [&](int r, int ty, int a0, int a1) { put(s_depth[r], (uint32_t)r, ty, a0, a1); });
+    }
 }
 
 cudaError_t launch_emit(const WsPtrs &ws, const Dims &d, cudaStream_t st) {
-    const uint32_t cells = (uint32_t)d.V * (uint32_t)d.nblk;
-    const cudaError_t e = launch_dep(k_emit, dim3(cells * (uint32_t)(kCell / kEmitThreads) + kBigBlocks),
-                                     dim3(kEmitThreads), st, ws, d);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    const cudaError_t e = launch_dep(k_emit, dim3((uint32_t)d.V * (uint32_t)d.nblk), dim3(kBlock), st, ws, d);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace gsk
