@@ -207,8 +207,8 @@ def _ptr(t) -> int | None:
 
 
 def _stream(stream) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:  # the raw handle: building a torch.cuda.Stream costs 4 us a call
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -662,13 +662,19 @@ class Rasterizer:
         self._keep = [g, poses, targets]
         return out
 
+    def _zero_grads(self, g: GaussianTensors) -> dict:
+        """FP32 gradients of g's parameters, zero (one launch for all of them)."""
+        grads = {k: torch.empty(getattr(g, k).shape, dtype=torch.float32, device=self.device)
+                 for k in ("means", "quats", "log_scales", "logits", "rgb") if getattr(g, k) is not None}
+        torch._foreach_zero_(list(grads.values()))
+        return grads
+
     def backward(self, g: GaussianTensors, upstream=None, params: bool = True, pose: bool = True,
                  stream=None, n_views: int = 1) -> dict:
         out = {}
         grads = None
         if params:
-            out["grads"] = {k: torch.zeros(getattr(g, k).shape, dtype=torch.float32, device=self.device)
-                            for k in ("means", "quats", "log_scales", "logits", "rgb") if getattr(g, k) is not None}
+            out["grads"] = self._zero_grads(g)
             G = out["grads"]
             grads = gs_gaussians_grad(_ptr(G["means"]), _ptr(G.get("quats")), _ptr(G["log_scales"]), _ptr(G["logits"]),
                                       _ptr(G["rgb"]))
@@ -688,8 +694,7 @@ class Rasterizer:
         depth HW, prior HW or None) device tensors.  Returns {'grads': ..., 'loss': V}."""
         V = len(cams)
         if grads is None:
-            grads = {k: torch.zeros(getattr(g, k).shape, dtype=torch.float32, device=self.device)
-                     for k in ("means", "quats", "log_scales", "logits", "rgb") if getattr(g, k) is not None}
+            grads = self._zero_grads(g)
         G = gs_gaussians_grad(_ptr(grads["means"]), _ptr(grads.get("quats")), _ptr(grads["log_scales"]),
                               _ptr(grads["logits"]), _ptr(grads["rgb"]))
         loss = torch.zeros(V, dtype=torch.float64, device=self.device)
