@@ -181,18 +181,24 @@ struct GaussPtrs {
     const void *quats, *log_scales, *logits, *rgb;
 };
 
-// Pair counters of a tile block: every warp adds its lanes' counts to the block's shared
-// totals (zeroed before the block's first barrier), and one thread adds those to the header
-// after the block's last barrier.
-__device__ __forceinline__ void count_warp(uint32_t evals, uint32_t contrib, unsigned long long *s_count) {
+// Pair counters of a tile block: every warp posts its lanes' sums, and one thread adds
+// them to the header after the block's last barrier.
+__device__ __forceinline__ void count_warp(uint32_t evals, uint32_t contrib, uint2 *s_count) {
     const uint32_t we = __reduce_add_sync(0xffffffffu, evals), wc = __reduce_add_sync(0xffffffffu, contrib);
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(s_count, (unsigned long long)we);
-        atomicAdd(s_count + 1, (unsigned long long)wc);
-    }
+    if ((threadIdx.x & 31) == 0) s_count[threadIdx.x >> 5] = make_uint2(we, wc);
 }
 __device__ __forceinline__ void red_add64(unsigned long long *p, unsigned long long v) {
     asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+__device__ __forceinline__ void count_block(const uint2 *s_count, unsigned long long *evals, unsigned long long *contrib) {
+    unsigned long long e = 0, c = 0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        e += s_count[w].x;
+        c += s_count[w].y;
+    }
+    red_add64(evals, e);
+    red_add64(contrib, c);
 }
 
 // Fire-and-forget global add (no value returned, so the thread does not wait for it).
@@ -539,12 +545,18 @@ __device__ __forceinline__ int build_patch_list(const float4 *sBox, const float4
     return nl;
 }
 
-// Global tile -> view (binary search over the views' first tiles).
+// Global tile -> view, by a whole warp: the views' first tiles are probed 32 at a time (one
+// load for up to 32 views, two for 1,024), so a tile block finds its view without a chain of
+// dependent loads by one thread and a barrier.
 __device__ __forceinline__ int view_of_tile(const ViewInfo *views, int V, uint32_t tile) {
-    int lo = 0, hi = V - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (views[mid].tile_base <= tile) lo = mid; else hi = mid - 1;
+    const int lane = threadIdx.x & 31;
+    int lo = 0, len = V;
+    while (len > 1) {
+        const int step = (len + 31) / 32, at = lane * step;
+        const bool le = at < len && views[lo + at].tile_base <= tile;
+        const int k = __popc(__ballot_sync(0xffffffffu, le)) - 1;  // the first is never above
+        lo += k * step;
+        len = min(step, len - k * step);
     }
     return lo;
 }

@@ -57,19 +57,12 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
     __shared__ __align__(16) uint16_t sList[kTilePix / 32][NB];  // byte offsets: 16 x batch position
     __shared__ float sAcc[NB * A::kStride];
     __shared__ __align__(16) float sRows[kTilePix / 32][kWalkFloats<true>];  // the reverse walk's transposed rows
-    __shared__ int s_view;
     __shared__ float s_loss[kTilePix / 32];
-    __shared__ uint32_t s_nmax;
-    __shared__ unsigned long long s_count[4];
+    __shared__ uint32_t s_last[kTilePix / 32];
+    __shared__ uint2 s_fwd[kTilePix / 32], s_rev[kTilePix / 32];
     const uint32_t tile = L.ws.tile_order[blockIdx.x];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) {
-        s_view = view_of_tile(L.ws.views, L.d.V, tile);
-        s_nmax = 0;
-    }
-    if (tid < 4) s_count[tid] = 0ull;
-    __syncthreads();
-    const ViewInfo vi = L.ws.views[s_view];
+    const ViewInfo vi = L.ws.views[view_of_tile(L.ws.views, L.d.V, tile)];
     const uint32_t local = tile - vi.tile_base;
     const int tx = (int)(local % (uint32_t)vi.tiles_x), ty = (int)(local / (uint32_t)vi.tiles_x);
     constexpr int kPPR = (1 << LW) / kPatchW;  // 8 x 4 patches per patch row (tile width 2^LW)
@@ -102,7 +95,7 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
     int64_t staged = -1;  // first list entry of the batch now in shared memory (block-uniform)
     int nl_staged = 0;    // length of this warp's list of the staged batch (warp-uniform)
     for (uint32_t b0 = 0; b0 < n; b0 += NB) {
-        if (__syncthreads_count(!walk.done) == 0) break;
+        if (b0 && __syncthreads_count(!walk.done) == 0) break;  // (and all have walked the staged batch)
         const uint32_t idx = b0 + tid;
         if (tid < NB && idx < n) stage_one(L, L.ws.sorted[start + idx], x0, y0, sP0, sP1, sC, sBox, tid);
         staged = b0;
@@ -135,7 +128,7 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
     const float cr = walk.cr, cg = walk.cg, cb = walk.cb, D = walk.D;
     uint32_t last = walk.last;
     const float Sil = 1.f - T;  // Eq. 4 summed: 1 - prod(1 - a_i)
-    count_warp(n_eval, n_contrib, s_count);
+    count_warp(n_eval, n_contrib, s_fwd);
 
     // ---------------------------------------------------------------- fused loss
     if (!targets_loaded && inside) {  // an empty tile list: no batch was staged
@@ -181,11 +174,9 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
     // the reverse walk evaluates this pixel's entries in front of its last contributor and
     // differentiates its contributions: the forward's counts up to that entry
     const uint32_t rev_eval = last ? walk.eval_last : 0u, rev_contrib = last ? n_contrib : 0u;
-    count_warp(rev_eval, rev_contrib, s_count + 2);
-    uint32_t wlast = last;  // largest contributor count in the warp
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) wlast = max(wlast, __shfl_xor_sync(0xffffffffu, wlast, off));
-    if (lane == 0 && wlast) atomicMax(&s_nmax, wlast);
+    count_warp(rev_eval, rev_contrib, s_rev);
+    const uint32_t wlast = __reduce_max_sync(0xffffffffu, last);  // largest contributor count in the warp
+    if (lane == 0) s_last[warp] = wlast;
     const PixUp up{g0, g1, g2, gD, gS};
     float *buf = sRows[warp];
     store_planes<true>(buf, up, lane);
@@ -197,7 +188,7 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
         const bool resident = b0 == staged;
         const uint32_t filled = min((uint32_t)NB, n - (uint32_t)b0);
         if (!resident) {
-            __syncthreads();  // the flush of the batch behind has read the sums
+            // (thread tid flushed the row it clears here, and the others walk no more)
             if (tid < filled) stage_one(L, L.ws.sorted[start + (uint32_t)b0 + tid], x0, y0, sP0, sP1, sC, sBox, tid);
             if (tid < NB) {
 #pragma unroll
@@ -229,7 +220,8 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
         bwd_walk_batch<true, false>(sList[warp], nl, lim, sP0, sP1, sC, uv, pu_lo, pv_lo, thr, S.alpha_max, up, T, GB,
                                     buf, sAcc, lane, unused, unused);
         __syncthreads();
-        const uint32_t nmax = s_nmax;
+        uint32_t nmax = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) nmax = max(nmax, s_last[w]);
         if (nmax > (uint32_t)b0 && tid < min(filled, nmax - (uint32_t)b0)) {
             const uint32_t r = L.ws.sorted[start + (uint32_t)b0 + tid];
             if (r < rec_slots(L.d)) flush_acc<true>(sAcc + tid * A::kStride, L.ws.rec[r].b, 1.f, L.ws.rec_grad + r);
@@ -240,10 +232,8 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
         DF s{0.f, 0.f};
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s = df_add(s, DF{s_loss[w], 0.f});
         L.ws.tile_loss[tile] = df_pack(s);
-        red_add64(&L.ws.hdr->fwd_evals, s_count[0]);
-        red_add64(&L.ws.hdr->fwd_contrib, s_count[1]);
-        red_add64(&L.ws.hdr->bwd_evals, s_count[2]);
-        red_add64(&L.ws.hdr->bwd_contrib, s_count[3]);
+        count_block(s_fwd, &L.ws.hdr->fwd_evals, &L.ws.hdr->fwd_contrib);
+        count_block(s_rev, &L.ws.hdr->bwd_evals, &L.ws.hdr->bwd_contrib);
     }
 }
 

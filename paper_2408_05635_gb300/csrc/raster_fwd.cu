@@ -35,19 +35,11 @@ __global__ void __launch_bounds__(kTilePix, 5) k_forward(ForwardLaunch L) {
     __shared__ float4 sP0[NB], sC[NB], sBox[NB];
     __shared__ float4 sP1[NB];                     // (kuu, lo, -1/(2 kuu), -1/(2 kvv)): the stride of sP0, sC
     __shared__ __align__(16) uint16_t sList[kTilePix / 32][NB];  // byte offsets: 16 x batch position
-    __shared__ int s_view;
     __shared__ float s_loss[kTilePix / 32];
-    __shared__ unsigned long long s_count[2];
+    __shared__ uint2 s_count[kTilePix / 32];
     const uint32_t tile = L.ws.tile_order[blockIdx.x];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) {
-        s_view = view_of_tile(L.ws.views, L.d.V, tile);
-        s_count[0] = s_count[1] = 0ull;
-    }
-    __syncthreads();
-    const int view = s_view;
-    (void)view;
-    const ViewInfo vi = L.ws.views[view];
+    const ViewInfo vi = L.ws.views[view_of_tile(L.ws.views, L.d.V, tile)];
     const uint32_t local = tile - vi.tile_base;
     const int tx = (int)(local % (uint32_t)vi.tiles_x), ty = (int)(local / (uint32_t)vi.tiles_x);
     constexpr int kPPR = (1 << LW) / kPatchW;  // 8 x 4 patches per patch row (tile width 2^LW)
@@ -85,7 +77,7 @@ __global__ void __launch_bounds__(kTilePix, 5) k_forward(ForwardLaunch L) {
         }
     };
     for (uint32_t b0 = 0; b0 < n; b0 += NB) {
-        if (__syncthreads_count(!walk.done) == 0) break;
+        if (b0 && __syncthreads_count(!walk.done) == 0) break;  // (and all have walked the staged batch)
         const uint32_t idx = b0 + tid;
         if (tid < NB && idx < n) {  // thread tid stages batch position tid
             const uint32_t r = L.ws.sorted[start + idx];
@@ -180,8 +172,7 @@ __global__ void __launch_bounds__(kTilePix, 5) k_forward(ForwardLaunch L) {
             for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s = df_add(s, DF{s_loss[w], 0.f});
             L.ws.tile_loss[tile] = df_pack(s);
         }
-        red_add64(&L.ws.hdr->fwd_evals, s_count[0]);
-        red_add64(&L.ws.hdr->fwd_contrib, s_count[1]);
+        count_block(s_count, &L.ws.hdr->fwd_evals, &L.ws.hdr->fwd_contrib);
     }
 }
 
