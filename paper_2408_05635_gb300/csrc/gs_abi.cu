@@ -41,7 +41,7 @@ uint32_t max_sub(uint64_t T) {
 
 struct Layout {
     size_t err, hdr, tile_cnt, zero_end;
-    size_t views, view_rt, cell_cnt, tile_start, cursor, tile_order, rec, rec_grad, keys, sorted, t_final, n_last,
+    size_t views, view_rt, cell_cnt, tile_start, cursor, tile_order, rec, rec_grad, keys, sorted, hits, t_final, n_last,
         upstream, tile_loss, pose_part, rkeys, rvals, rhist, rtotal, scan_part, total;
 };
 
@@ -307,6 +307,7 @@ gs_status build_problem(gs_ctx *ctx, const gs_problem *p, Problem &out) {
     L.rec_grad = take(sizeof(RecGrad) * cells * kCell);
     L.keys = take(sizeof(unsigned long long) * (size_t)d.pair_cap);
     L.sorted = take(sizeof(uint32_t) * (size_t)d.pair_cap);
+    L.hits = take(sizeof(uint32_t) * (kTilePix / 32) * ((size_t)d.pair_cap / 32 + (size_t)lay_tiles + 1));
     L.t_final = take(sizeof(float) * (size_t)d.P);
     L.n_last = take(sizeof(uint32_t) * (size_t)d.P);
     L.upstream = take(sizeof(float) * 5 * (size_t)d.P);
@@ -338,6 +339,7 @@ WsPtrs ws_ptrs(void *base, const Layout &L) {
     w.rec_grad = reinterpret_cast<RecGrad *>(b + L.rec_grad);
     w.keys = reinterpret_cast<unsigned long long *>(b + L.keys);
     w.sorted = reinterpret_cast<uint32_t *>(b + L.sorted);
+    w.hits = reinterpret_cast<uint32_t *>(b + L.hits);
     w.t_final = reinterpret_cast<float *>(b + L.t_final);
     w.n_last = reinterpret_cast<uint32_t *>(b + L.n_last);
     w.upstream = reinterpret_cast<float *>(b + L.upstream);

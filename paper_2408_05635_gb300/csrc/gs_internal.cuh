@@ -126,6 +126,7 @@ struct WsPtrs {
     RecGrad *rec_grad;     // same slots
     unsigned long long *keys;  // pair_capacity
     uint32_t *sorted;      // pair_capacity, record ids in (tile, depth, gaussian) order
+    uint32_t *hits;        // the warps' hit words of every tile (hit_words), or nullptr (a forward alone)
     float *t_final;        // P, transmittance after the last contributor
     uint32_t *n_last;      // P, tile-list index + 1 of the last contributor
     float *upstream;       // 5 x P: dL/dC (planar like the images), dL/dD, dL/dS of the fused loss
@@ -157,7 +158,7 @@ struct Dims {
     int32_t nblk;          // ceil(n / kBlock): cells per view
     uint32_t T;            // tiles over all views
     uint32_t S;            // sub-buckets per tile (1, 2 or 4): a tile's pairs are counted and
-                           // placed through S counters picked by Gaussian index, so no single
+                           // placed through S counters picked by cell, so no single
                            // counter takes every pair of a crowded tile; the S sub-ranges are
                            // contiguous, so the tile's list is still one range
     uint32_t P;            // pixels over all views
@@ -524,11 +525,15 @@ __device__ __forceinline__ float2 p1_at(const float4 *sP1, int off) {
 // A warp's list of the batch positions [0, cnt) whose footprint reaches its pixel
 // rectangle [pu_lo, pu_hi] x [pv_lo, pv_hi]: the support box first, then the exact
 // footprint test; entries are byte offsets (16 x position) in ascending order.  Returns
-// the count (warp-uniform).
+// the count (warp-uniform).  keep(word): called once at the end by the lanes below
+// ceil(cnt / 32), each with the 32 hits of its ballot, for the reverse walk
+// (list_from_words).
+template <class Keep>
 __device__ __forceinline__ int build_patch_list(const float4 *sBox, const float4 *sP0, const float4 *sP1,
                                                 uint16_t *list, int cnt, int lane, float thr, float pu_lo,
-                                                float pu_hi, float pv_lo, float pv_hi) {
+                                                float pu_hi, float pv_lo, float pv_hi, Keep &&keep) {
     int nl = 0;
+    uint32_t kept = 0;  // ballot `lane`
     for (int k = 0; k < cnt; k += 32) {
         const int j = k + lane;
         bool hit = false;
@@ -538,11 +543,35 @@ __device__ __forceinline__ int build_patch_list(const float4 *sBox, const float4
             if (hit) hit = footprint_meets_rect(sP0[j], sP1[j], thr, pu_lo, pu_hi, pv_lo, pv_hi);
         }
         const uint32_t m = __ballot_sync(0xffffffffu, hit);
+        if (lane == k >> 5) kept = m;
         if (hit) list[nl + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(j << 4);
+        nl += __popc(m);
+    }
+    if (32 * lane < cnt) keep(kept);
+    __syncwarp();
+    return nl;
+}
+
+// The same list from the hit words the forward kept: w holds word `lane` of the batch.  The
+// forward's test took 45 instructions per 32 candidates and warp, a tenth of the reverse
+// walk's.
+__device__ __forceinline__ int list_from_words(uint32_t w, uint16_t *list, int cnt, int lane) {
+    int nl = 0;
+    for (int k = 0; k < cnt; k += 32) {
+        uint32_t m = __shfl_sync(0xffffffffu, w, k >> 5);
+        if (cnt - k < 32) m &= (1u << (cnt - k)) - 1u;
+        if ((m >> lane) & 1u) list[nl + __popc(m & ((1u << lane) - 1u))] = (uint16_t)((k + lane) << 4);
         nl += __popc(m);
     }
     __syncwarp();
     return nl;
+}
+
+// A warp's hit words of its tile (n > 0 entries from `start`), one bit per list entry.  Tiles
+// start at word 8 (start / 32 + tile): with the lists' starts ascending with the tile, each
+// has room for the ceil(n / 32) words of its up to eight warps.
+__device__ __forceinline__ uint32_t *hit_words(const WsPtrs &ws, uint32_t tile, uint32_t start, uint32_t n, int warp) {
+    return ws.hits + (size_t)((start >> 5) + tile) * (kTilePix / 32) + (size_t)warp * ((n + 31u) >> 5);
 }
 
 // Global tile -> view, by a whole warp: the views' first tiles are probed 32 at a time (one

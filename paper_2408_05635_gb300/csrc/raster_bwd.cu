@@ -19,8 +19,8 @@
 // Batches of NB records (64, 128 or 256, the batch depth, picked per context) are staged
 // by the first NB threads, from the tile's last contributor backwards.  Each warp owns an
 // 8 x 4 patch of the tile and walks, back to front, only the staged Gaussians whose
-// footprint can reach alpha_min on the patch (build_patch_list) and that precede its last
-// contributor.
+// footprint can reach alpha_min on the patch (the hits the forward kept) and that precede its
+// last contributor.
 // Reduction: each warp sums its 32 pixels' terms of eight Gaussians at a time through a
 // small shared matrix read transposed (bwd_walk.cuh), adds the sums into a per-batch
 // shared-memory accumulator, and the block flushes once per (tile, Gaussian) with vector
@@ -29,6 +29,9 @@
 // block's start; the view is found by each warp, a one-batch list is staged beside the
 // pixels' loads, and a thread owns its batch position up to the flush (two barriers a batch
 // instead of three): 1,204 -> 1,139 us on the mapping window, 411 -> 387 on the dense one.
+// The lists come from the forward's hit words (8 words a warp and batch instead of 256 tests):
+// 1,139 -> 1,083 and 387 -> 358 us, the forward 739 -> 747 (it keeps them for every render,
+// since a reverse walk may follow: 113 -> 115 us on 1M at 1200 x 680).
 // Lanes whose pixel the Gaussian does not reach take a = 0, which leaves T and g.B
 // unchanged and zeroes every term, so the walk has no divergent branch.
 #include "gs_internal.cuh"
@@ -46,8 +49,8 @@ __global__ void __launch_bounds__(kTilePix, 4) k_backward(BackwardLaunch L) {
     griddep_launch_dependents();
     using A = Acc<POSE>;
     extern __shared__ __align__(16) float sDyn[];
-    __shared__ float4 sP0[NB], sC[NB], sBox[NB];
-    __shared__ float4 sP1[NB];  // (kuu, lo, -1/(2 kuu), -1/(2 kvv)): the stride of sP0, sC
+    __shared__ float4 sP0[NB], sC[NB];
+    __shared__ float4 sP1[NB];  // (kuu, lo, -, -): the stride of sP0, sC
     __shared__ float sAcc[NB * A::kStride];
     __shared__ __align__(16) uint16_t sList[kTilePix / 32][NB];  // byte offsets: 16 x batch position
     __shared__ uint32_t s_last[kTilePix / 32];
@@ -64,8 +67,7 @@ __global__ void __launch_bounds__(kTilePix, 4) k_backward(BackwardLaunch L) {
     const bool inside = px < vi.width && py < vi.height;
     const float x0 = (float)(tx << LW), y0 = (float)(ty << vi.tile_lh);
     const float2 uv = make_float2((float)lu, (float)lv);  // tile-local pixel centre
-    const float pu_lo = (float)pu0, pu_hi = (float)(pu0 + kPatchW - 1);
-    const float pv_lo = (float)pv0, pv_hi = (float)(pv0 + kPatchH - 1);
+    const float pu_lo = (float)pu0, pv_lo = (float)pv0;
     const Settings &S = L.s;
     const float thr = S.log2_alpha_min;
     float *buf = sDyn + warp * kWalkFloats<POSE>;
@@ -83,12 +85,10 @@ __global__ void __launch_bounds__(kTilePix, 4) k_backward(BackwardLaunch L) {
                 const Rec rr = L.ws.rec[r];
                 const Footprint f = stage_footprint(rr.a, rr.b, x0, y0);
                 sP0[tid] = f.p0;
-                sP1[tid] = f.p1;
+                sP1[tid] = make_float4(f.p1.x, f.p1.y, 0.f, 0.f);
                 sC[tid] = make_float4(rr.c.x, rr.c.y, rr.c.z, rr.a.z);
-                sBox[tid] = stage_box(rr.b, -f.p0.x, -f.p0.y);
             } else {
-                sBox[tid] = make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY);
-                r = ~0u;
+                r = ~0u;  // none: the forward kept no hit of it
             }
         }
         if (tid < NB) {
@@ -100,6 +100,10 @@ __global__ void __launch_bounds__(kTilePix, 4) k_backward(BackwardLaunch L) {
     // a list of one batch is staged before the pixels' last contributors are known, its
     // loads beside theirs
     const bool single = n <= (uint32_t)NB;
+    const auto load_words = [&](uint32_t first) {  // this warp's hits of the batch, a word per lane
+        return lane < NB / 32 && first + 32u * lane < n ? hit_words(L.ws, tile, start, n, warp)[(first >> 5) + lane] : 0u;
+    };
+    uint32_t hits = single ? load_words(0u) : 0u;
     uint32_t rec = single ? stage(0u, (int)n) : ~0u;
     const uint32_t HW = (uint32_t)vi.width * (uint32_t)vi.height;
     const uint32_t p = (uint32_t)py * (uint32_t)vi.width + (uint32_t)px;
@@ -133,12 +137,13 @@ __global__ void __launch_bounds__(kTilePix, 4) k_backward(BackwardLaunch L) {
     for (int64_t b0 = nmax ? (int64_t)((nmax - 1) / NB) * NB : -1; b0 >= 0; b0 -= NB) {
         const int cnt = (int)min((uint32_t)NB, nmax - (uint32_t)b0);
         if (!single) {
+            hits = load_words((uint32_t)b0);
             rec = stage((uint32_t)b0, cnt);
             __syncthreads();
         }
         // this warp's list, limited to entries below its largest contributor count
         const int wcnt = (int)min((int64_t)cnt, (int64_t)wlast - b0);
-        const int nl = build_patch_list(sBox, sP0, sP1, sList[warp], wcnt, lane, thr, pu_lo, pu_hi, pv_lo, pv_hi);
+        const int nl = list_from_words(hits, sList[warp], wcnt, lane);
         // entries at byte offsets below lim are in front of this pixel's last contributor
         const int lim = (int)max(min((int64_t)last - b0, (int64_t)NB), (int64_t)0) * 16;
         bwd_walk_batch<POSE, true>(sList[warp], nl, lim, sP0, sP1, sC, uv, pu_lo, pv_lo, thr, S.alpha_max, up, T, GB,

@@ -117,7 +117,11 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
         }
         const int cnt = (int)min((uint32_t)NB, n - b0);
         if (__any_sync(0xffffffffu, !walk.done)) {
-            const int nl = build_patch_list(sBox, sP0, sP1, sList[warp], cnt, lane, thr, pu_lo, pu_hi, pv_lo, pv_hi);
+            // (its hits kept where the reverse walk will stage the batch again)
+            const int nl = build_patch_list(sBox, sP0, sP1, sList[warp], cnt, lane, thr, pu_lo, pu_hi, pv_lo, pv_hi,
+                                            [&](uint32_t hits) {
+                                                if (n > (uint32_t)NB) hit_words(L.ws, tile, start, n, warp)[(b0 >> 5) + lane] = hits;
+                                            });
             nl_staged = nl;
             if (!walk.done)
                 fwd_walk_batch(walk, sList[warp], nl, b0, sP0, sP1, sC, uv, thr, S.alpha_max, S.t_min, n_eval,
@@ -187,7 +191,10 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
     for (int64_t b0 = staged; b0 >= 0; b0 -= NB) {
         const bool resident = b0 == staged;
         const uint32_t filled = min((uint32_t)NB, n - (uint32_t)b0);
+        uint32_t words = 0;
         if (!resident) {
+            // this warp's hits (it kept them for every batch its pixels reached)
+            if (lane < NB / 32 && b0 < (int64_t)wlast) words = hit_words(L.ws, tile, start, n, warp)[(b0 >> 5) + lane];
             // (thread tid flushed the row it clears here, and the others walk no more)
             if (tid < filled) stage_one(L, L.ws.sorted[start + (uint32_t)b0 + tid], x0, y0, sP0, sP1, sC, sBox, tid);
             if (tid < NB) {
@@ -211,7 +218,7 @@ __global__ void __launch_bounds__(kTilePix, 4) k_track_tile(TrackTileLaunch L) {
                 if (m < 32) break;
             }
         } else {
-            nl = build_patch_list(sBox, sP0, sP1, sList[warp], wcnt, lane, thr, pu_lo, pu_hi, pv_lo, pv_hi);
+            nl = list_from_words(words, sList[warp], wcnt, lane);
         }
         __syncwarp();
         // entries at byte offsets below lim are in front of this pixel's last contributor

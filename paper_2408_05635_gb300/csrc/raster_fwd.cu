@@ -97,7 +97,11 @@ __global__ void __launch_bounds__(kTilePix, 5) k_forward(ForwardLaunch L) {
         const int cnt = (int)min((uint32_t)NB, n - b0);
         if (__any_sync(0xffffffffu, !walk.done)) {
             // this warp's list: the batch Gaussians whose footprint reaches its 8 x 4 patch
-            const int nl = build_patch_list(sBox, sP0, sP1, sList[warp], cnt, lane, thr, pu_lo, pu_hi, pv_lo, pv_hi);
+            // (its hits kept for the reverse walk)
+            const int nl = build_patch_list(sBox, sP0, sP1, sList[warp], cnt, lane, thr, pu_lo, pu_hi, pv_lo, pv_hi,
+                                            [&](uint32_t hits) {
+                                                if (L.ws.hits) hit_words(L.ws, tile, start, n, warp)[(b0 >> 5) + lane] = hits;
+                                            });
             if (!walk.done)
                 fwd_walk_batch(walk, sList[warp], nl, b0, sP0, sP1, sC, uv, thr, S.alpha_max, S.t_min, n_eval,
                                n_contrib);
