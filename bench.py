@@ -767,8 +767,11 @@ def ncu_traffic(kernel):
             f = line.split()
             if len(f) >= 5 and f[0] == "traffic" and f[1] == kernel:
                 h = hashlib.sha256()
-                for src in f[4:]:
-                    h.update(open(os.path.join(root, "paper_2408_05635_gb300", "csrc", src), "rb").read())
+                srcs = [os.path.join(root, "paper_2408_05635_gb300", "csrc", src) for src in f[4:]]
+                if not all(os.path.exists(src) for src in srcs):  # renamed or gone: not the sources measured
+                    return None, os.path.relpath(path, root)
+                for src in srcs:
+                    h.update(open(src, "rb").read())
                 return (int(f[2]) if h.hexdigest()[:16] == f[3] else None), os.path.relpath(path, root)
     return None, None
 
