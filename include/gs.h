@@ -482,7 +482,9 @@ gs_status gs_map_prune(const gs_map_config *cfg, const gs_map *src, const int64_
  * rgb_t / depth_t: the observation, planar FP32 device arrays of `pixels` pixels; out:
  * device, 4 doubles = (sum of squared colour errors over every pixel and channel,
  * sum |D - D*| over the pixels with D* > 0, their count, sum (D - D*)^2 over them),
- * accumulated in FP64 in a fixed order.  Errors: INVALID_ARG, CUDA. */
+ * in a fixed order (for a given device) with at least the precision of FP64 accumulation:
+ * FP64 across groups of eight threads, three FP32 values with their rounding errors inside
+ * them.  Errors: INVALID_ARG, CUDA. */
 gs_status gs_image_metrics(const float *rgb, const float *depth, const float *rgb_t, const float *depth_t,
                            int64_t pixels, double *out, void *stream);
 
