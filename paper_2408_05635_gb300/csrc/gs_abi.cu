@@ -1177,18 +1177,22 @@ gs_status gs_sync_status(gs_ctx *ctx, void *stream, gs_counts *counts) {
     ctx->err.clear();
     if (!ctx->bound) return fail(ctx, GS_ERR_STATE, "no workspace bound");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // the flags and the header in one copy on the stream into page-locked memory, and one
-    // wait (a wait and two copies into pageable memory took the host 25 us longer)
+    // the flags and the header in one copy into page-locked memory and one wait (a wait and two
+    // copies into pageable memory took the host 25 us longer).  The copy is on the legacy
+    // default stream, so that it also follows work of the caller's that is still running there
+    // or on a blocking stream when `stream` is another one; that one is waited for first.
     const size_t span = (size_t)(reinterpret_cast<char *>(ctx->ws.hdr + 1) - reinterpret_cast<char *>(ctx->ws.err));
     cudaError_t e = cudaSuccess;
+    if (s && s != cudaStreamLegacy && (e = cudaStreamSynchronize(s)) != cudaSuccess)
+        return cuda_fail(ctx, e, "stream synchronize");
     if (!ctx->status_host && (e = cudaMallocHost(&ctx->status_host, kStatusBytes)) != cudaSuccess) {
         ctx->status_host = nullptr;
         return cuda_fail(ctx, e, "status buffer");
     }
     if (span > kStatusBytes) return fail(ctx, GS_ERR_STATE, "workspace header layout");
-    if ((e = cudaMemcpyAsync(ctx->status_host, ctx->ws.err, span, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+    if ((e = cudaMemcpyAsync(ctx->status_host, ctx->ws.err, span, cudaMemcpyDeviceToHost, cudaStreamLegacy)) != cudaSuccess)
         return cuda_fail(ctx, e, "status read");
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(ctx, e, "stream synchronize");
+    if ((e = cudaStreamSynchronize(cudaStreamLegacy)) != cudaSuccess) return cuda_fail(ctx, e, "stream synchronize");
     DevHeader h;
     uint32_t err;
     std::memcpy(&h, static_cast<const char *>(ctx->status_host) + span - sizeof(h), sizeof(h));
