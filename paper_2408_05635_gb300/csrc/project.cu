@@ -45,11 +45,25 @@ __device__ __forceinline__ bool record_rect(const ViewInfo &vi, float4 A, float4
 // of 1M Gaussians (29 pairs a record): k_project 185 -> 113 us, k_emit 161 -> 74; one view
 // of 1M at 1200 x 680 (10 pairs): 48 -> 29 and 64 -> 38; 2M in FP16 (4.6): 80 -> 63 and 87
 // -> 40 (k_emit's times hold its wait for the scan).  Unchanged within a microsecond where
-// latency counts (200k, 37k records) and on footprints a pixel wide (1.8 pairs a record: 57
-// -> 61 and 61 -> 55 us).
+// latency counts (200k, 37k records); footprints a pixel wide (1.8 pairs a record) 57 -> 61 and 61 -> 55 us.
+//
+// The box pays where records share its tiles.  Where the tiles are many more than the records
+// could meet, zeroing and reading them back costs more than an atomic a pair: 1M pixel-sized
+// Gaussians in random order at 1200 x 680 (a block's box is the image) took 143 us a projection
+// with it, 108 without; of six pixels (6 tiles a rectangle, so 2.1 box tiles a tile) 63 against 78.
+// Without it a record's rows are walked as they are, or, where rows are wide, by four or eight
+// threads each, whose atomics fall on neighbouring counters: 200k Gaussians of 40 pixels in
+// random order at 1920 x 1080 took 1,376 us with a thread a row, 905 with eight (982 with a
+// warp a record); of ten pixels 172 and 150 with four.
 constexpr int kSoloRows = 4;     // records of no more rows: handing their rows out costs more than walking them
                                  // (1.8 pairs a record: a window of 864 us took 887)
-constexpr int kBoxTiles = 3328;  // a 1200 x 680 image has 3,225 tiles; beyond, atomics go to global memory
+constexpr int kBoxPerTile = 3;   // most tiles of a box per tile of its records' rectangles
+// Most tiles of a box, by the shared memory of six blocks an SM; k_emit's is smaller because its
+// scattered loads and stores want the L1 that is left (1M two-pixel Gaussians in random order:
+// 53 us, and 65 with 4,864; k_project's 58 with either, and 200k of 40 pixels over 4,800 tiles
+// 205 -> 52).
+constexpr int kProjectBox = 5632;
+constexpr int kEmitBox = 3328;
 
 struct RowRec {  // one record's rows
     float4 a;    // mu'_x, mu'_y, b, det
@@ -58,31 +72,42 @@ struct RowRec {  // one record's rows
     int tx0, tx1, ty0;
 };
 
-struct BinSmem {
+struct BinRows {
     RowRec rec[kBlock];
     uint32_t pre[kBlock + 1];  // rows before each record
-    uint32_t box[kBoxTiles];
     int4 warp_box[kWarps];     // first tile column and row, last column and row
-    uint2 warp_rows[kWarps];   // rows, and the most of one record
+    uint4 warp_rows[kWarps];   // rows, the most of one record, tiles of the rectangles
 };
 
-// Posts the warp's rows and tile box (block_box reads them after a barrier); returns the rows
-// of the warp's lanes before this one.
-__device__ __forceinline__ uint32_t post_rows(BinSmem &sm, bool has, int tx0, int tx1, int ty0, int ty1) {
+template <int TILES>
+struct BinSmem : BinRows {
+    uint32_t box[TILES];
+};
+
+// Posts the warp's rows and tile box (block_box reads them after a barrier).
+__device__ __forceinline__ void post_rows(BinRows &sm, bool has, int tx0, int tx1, int ty0, int ty1) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t rows = has ? (uint32_t)(ty1 - ty0 + 1) : 0u;
+    const uint32_t sum = __reduce_add_sync(0xffffffffu, rows);
+    const int lx = __reduce_min_sync(0xffffffffu, has ? tx0 : 0x7fffffff), hx = __reduce_max_sync(0xffffffffu, has ? tx1 : -1);
+    const int ly = __reduce_min_sync(0xffffffffu, has ? ty0 : 0x7fffffff), hy = __reduce_max_sync(0xffffffffu, has ? ty1 : -1);
+    const uint32_t most = __reduce_max_sync(0xffffffffu, rows);
+    const uint32_t tiles = __reduce_add_sync(0xffffffffu, has ? rows * (uint32_t)(tx1 - tx0 + 1) : 0u);
+    if (lane == 31) {
+        sm.warp_box[warp] = make_int4(lx, ly, hx, hy);
+        sm.warp_rows[warp] = make_uint4(sum, most, tiles, 0u);
+    }
+}
+
+// Rows of the warp's lanes before this one.
+__device__ __forceinline__ uint32_t rows_before(bool has, int ty0, int ty1) {
+    const int lane = threadIdx.x & 31;
     const uint32_t rows = has ? (uint32_t)(ty1 - ty0 + 1) : 0u;
     uint32_t incl = rows;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
         const uint32_t v = __shfl_up_sync(0xffffffffu, incl, off);
         if (lane >= off) incl += v;
-    }
-    const int lx = __reduce_min_sync(0xffffffffu, has ? tx0 : 0x7fffffff), hx = __reduce_max_sync(0xffffffffu, has ? tx1 : -1);
-    const int ly = __reduce_min_sync(0xffffffffu, has ? ty0 : 0x7fffffff), hy = __reduce_max_sync(0xffffffffu, has ? ty1 : -1);
-    const uint32_t most = __reduce_max_sync(0xffffffffu, rows);
-    if (lane == 31) {
-        sm.warp_box[warp] = make_int4(lx, ly, hx, hy);
-        sm.warp_rows[warp] = make_uint2(incl, most);
     }
     return incl - rows;
 }
@@ -91,29 +116,35 @@ struct BlockBox {
     int x, y, w, area;      // first tile, columns, tiles (0: gathered in global memory)
     bool boxed, solo;
     uint32_t before, rows;  // rows of the warps before this one, of the block
+    uint32_t lanes;         // threads that share a row (1, 4 or 8)
 };
 
-__device__ __forceinline__ BlockBox block_box(const BinSmem &sm) {
+__device__ __forceinline__ BlockBox block_box(const BinRows &sm, int most_tiles) {
     const int warp = threadIdx.x >> 5;
     int4 q = sm.warp_box[0];
-    uint2 r = sm.warp_rows[0];
+    uint4 r = sm.warp_rows[0];
     BlockBox o;
     o.before = warp > 0 ? r.x : 0u;
 #pragma unroll
     for (int w = 1; w < kWarps; ++w) {
         const int4 p = sm.warp_box[w];
-        const uint2 c = sm.warp_rows[w];
+        const uint4 c = sm.warp_rows[w];
         q = make_int4(min(q.x, p.x), min(q.y, p.y), max(q.z, p.z), max(q.w, p.w));
         o.before += w < warp ? c.x : 0u;
-        r = make_uint2(r.x + c.x, max(r.y, c.y));
+        r = make_uint4(r.x + c.x, max(r.y, c.y), r.z + c.z, 0u);
     }
     o.rows = r.x;
-    o.solo = r.y <= (uint32_t)kSoloRows;
     o.x = q.x;
     o.y = q.y;
     o.w = q.z - q.x + 1;
-    o.boxed = r.x > 0u && (int64_t)o.w * (q.w - q.y + 1) <= kBoxTiles;
-    o.area = o.boxed ? o.w * (q.w - q.y + 1) : 0;
+    const int64_t area = (int64_t)o.w * (q.w - q.y + 1);
+    o.boxed = r.x > 0u && area <= min((int64_t)most_tiles, (int64_t)kBoxPerTile * r.z);
+    o.area = o.boxed ? (int)area : 0;
+    // rows of three tiles on average by four threads, of twelve by eight: 200k Gaussians of ten
+    // pixels at 1280 x 720 (rows of 3) 412 -> 338 us with four, of 40 at 3840 x 2160 (28) 4,573
+    // with four and 3,225 with eight
+    o.lanes = o.boxed || r.z < 3u * r.x ? 1u : (r.z < 12u * r.x ? 4u : 8u);
+    o.solo = r.y <= (uint32_t)kSoloRows && o.lanes == 1u;
     return o;
 }
 
@@ -140,11 +171,11 @@ __device__ __forceinline__ void for_own_rows(const ViewInfo &vi, float4 A, float
 }
 
 // body(record, tile row, first tile column, last) for this thread's share of the rows of
-// nrec > 0 records.
+// nrec > 0 records, each row taken by `lanes` neighbouring threads.
 template <class Body>
-__device__ __forceinline__ void for_rows(const BinSmem &sm, int nrec, const ViewInfo &vi, Body &&body) {
+__device__ __forceinline__ void for_rows(const BinRows &sm, int nrec, const ViewInfo &vi, uint32_t lanes, Body &&body) {
     const uint32_t rows = sm.pre[nrec];
-    for (uint32_t f = threadIdx.x; f < rows; f += kBlock) {
+    for (uint32_t f = threadIdx.x / lanes; f < rows; f += kBlock / lanes) {
         int lo = 0, hi = nrec - 1;  // the last record whose prefix is at most f
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -586,7 +617,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_project(ProjectLaunch L) {
     __shared__ float sRt[12];
     __shared__ ViewInfo sv;
     __shared__ uint32_t warp_off[kWarps];
-    __shared__ BinSmem sm;
+    __shared__ BinSmem<kProjectBox> sm;
     const uint32_t cell = (uint32_t)v * (uint32_t)L.d.nblk + (uint32_t)b;
     if (tid == 0) {
         load_pose(L.poses + 7 * v, sRt);
@@ -704,7 +735,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_project(ProjectLaunch L) {
     // compaction into this block's cell: visible Gaussians take the first slots, in order
     const uint32_t ballot = __ballot_sync(0xffffffffu, vis);
     if (lane == 0) warp_off[warp] = __popc(ballot);
-    const uint32_t before = post_rows(sm, vis, tx0, tx1, ty0, ty1);
+    post_rows(sm, vis, tx0, tx1, ty0, ty1);
     __syncthreads();
     uint32_t nrec = 0, slot = __popc(ballot & ((1u << lane) - 1u));
 #pragma unroll
@@ -715,8 +746,9 @@ __global__ void __launch_bounds__(kBlock, 6) k_project(ProjectLaunch L) {
     }
     if (tid == 0) L.ws.cell_cnt[cell] = nrec;
     if (nrec == 0) return;
-    const BlockBox q = block_box(sm);
+    const BlockBox q = block_box(sm, kProjectBox);
     for (int k = tid; k < q.area; k += kBlock) sm.box[k] = 0u;
+    const uint32_t before = q.solo ? 0u : rows_before(vis, ty0, ty1);
     if (vis) {
         const uint32_t rec = cell * kCell + slot;
         Rec r;
@@ -730,22 +762,26 @@ __global__ void __launch_bounds__(kBlock, 6) k_project(ProjectLaunch L) {
             sm.pre[slot] = q.before + before;
         }
     }
-    if (tid == 0) sm.pre[nrec] = q.rows;
-    __syncthreads();
+    if (q.boxed || !q.solo) {
+        if (tid == 0) sm.pre[nrec] = q.rows;
+        __syncthreads();
+    }
     // pair counts per (tile, sub-bucket of the cell)
     uint32_t *cnt = L.ws.tile_cnt + vi.tile_base * L.d.S + ((uint32_t)b & (L.d.S - 1));
+    const int of_row = (int)((uint32_t)tid & (q.lanes - 1u));  // which of the row's threads this is
     const auto count = [&](int ty, int a0, int a1) {
         if (q.boxed) {
             uint32_t *row = sm.box + (ty - q.y) * q.w - q.x;
             for (int tx = a0; tx <= a1; ++tx) atomicAdd(row + tx, 1u);
         } else {
-            for (int tx = a0; tx <= a1; ++tx) red_add(cnt + (uint32_t)(ty * vi.tiles_x + tx) * L.d.S, 1u);
+            for (int tx = a0 + of_row; tx <= a1; tx += (int)q.lanes)
+                red_add(cnt + (uint32_t)(ty * vi.tiles_x + tx) * L.d.S, 1u);
         }
     };
     if (q.solo) {
         if (vis) for_own_rows(vi, A, B, tx0, tx1, ty0, ty1, count);
     } else {
-        for_rows(sm, (int)nrec, vi, [&](int, int ty, int a0, int a1) { count(ty, a0, a1); });
+        for_rows(sm, (int)nrec, vi, q.lanes, [&](int, int ty, int a0, int a1) { count(ty, a0, a1); });
     }
     if (!q.boxed) return;
     __syncthreads();
@@ -803,7 +839,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_emit(WsPtrs ws, Dims d) {
     const uint32_t cell = blockIdx.x;
     const int nrec = (int)ws.cell_cnt[cell];
     if (nrec == 0) return;
-    __shared__ BinSmem sm;
+    __shared__ BinSmem<kEmitBox> sm;
     __shared__ uint32_t s_depth[kBlock];
     const int tid = threadIdx.x;
     const int view = (int)(cell / (uint32_t)d.nblk);
@@ -817,31 +853,35 @@ __global__ void __launch_bounds__(kBlock, 6) k_emit(WsPtrs ws, Dims d) {
         B = rec.b;
         has = record_rect(vi, A, B, tx0, tx1, ty0, ty1);
     }
-    const uint32_t before = post_rows(sm, has, tx0, tx1, ty0, ty1);
+    post_rows(sm, has, tx0, tx1, ty0, ty1);
     __syncthreads();
-    const BlockBox q = block_box(sm);
+    const BlockBox q = block_box(sm, kEmitBox);
     for (int k = tid; k < q.area; k += kBlock) sm.box[k] = 0u;
+    const uint32_t before = q.solo ? 0u : rows_before(has, ty0, ty1);
     if (!q.solo && tid < nrec) {
         put_rows(sm.rec[tid], A, B, tx0, tx1, ty0);
         sm.pre[tid] = q.before + before;
         s_depth[tid] = __float_as_uint(A.z);
     }
-    if (tid == 0) sm.pre[nrec] = q.rows;
-    __syncthreads();
+    if (q.boxed || !q.solo) {
+        if (tid == 0) sm.pre[nrec] = q.rows;
+        __syncthreads();
+    }
     const bool radix = (d.flags & GS_SCHED_RADIX) != 0;
     const uint32_t sub = (cell % (uint32_t)d.nblk) & (d.S - 1), first = cell * kCell;
     const auto bucket_of = [&](int ty, int tx) { return (vi.tile_base + (uint32_t)(ty * vi.tiles_x + tx)) * d.S + sub; };
     if (!q.boxed) {
+        const int g = (int)q.lanes, of_row = tid & (g - 1);
         const auto emit = [&](uint32_t depth, uint32_t r, int ty, int a0, int a1) {
-            for (int t0 = a0; t0 <= a1; t0 += 4) {  // four atomics in flight before the stores
+            for (int t0 = a0 + of_row; t0 <= a1; t0 += 4 * g) {  // four atomics in flight before the stores
                 uint32_t slot[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    if (t0 + k <= a1) slot[k] = atomicAdd(ws.cursor + bucket_of(ty, t0 + k), 1u);
+                    if (t0 + k * g <= a1) slot[k] = atomicAdd(ws.cursor + bucket_of(ty, t0 + k * g), 1u);
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                    if (t0 + k <= a1) {
-                        const uint32_t bucket = bucket_of(ty, t0 + k);
+                    if (t0 + k * g <= a1) {
+                        const uint32_t bucket = bucket_of(ty, t0 + k * g);
                         if (slot[k] < ws.tile_start[bucket + 1] && slot[k] < d.pair_cap)
                             put_pair(ws, radix, slot[k], bucket / d.S, depth, first + r);
                         else
@@ -850,7 +890,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_emit(WsPtrs ws, Dims d) {
             }
         };
         if (!q.solo) {
-            for_rows(sm, nrec, vi, [&](int r, int ty, int a0, int a1) { emit(s_depth[r], (uint32_t)r, ty, a0, a1); });
+            for_rows(sm, nrec, vi, q.lanes, [&](int r, int ty, int a0, int a1) { emit(s_depth[r], (uint32_t)r, ty, a0, a1); });
         } else if (has) {
             for_own_rows(vi, A, B, tx0, tx1, ty0, ty1,
                          [&](int ty, int a0, int a1) { emit(__float_as_uint(A.z), (uint32_t)tid, ty, a0, a1); });
@@ -879,7 +919,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_emit(WsPtrs ws, Dims d) {
                 }
         }
     } else {
-        for_rows(sm, nrec, vi, [&](int, int ty, int a0, int a1) { count(ty, a0, a1); });
+        for_rows(sm, nrec, vi, 1u, [&](int, int ty, int a0, int a1) { count(ty, a0, a1); });
     }
     __syncthreads();
     for (int k0 = tid; k0 < q.area; k0 += 4 * kBlock) {  // counts to first slots, four tiles in flight
@@ -916,7 +956,7 @@ __global__ void __launch_bounds__(kBlock, 6) k_emit(WsPtrs ws, Dims d) {
         for (int k = 0; k < kSoloRows; ++k)
             put(__float_as_uint(A.z), (uint32_t)tid, ty0 + k, q.x + (int)(span[k] & 0xffffu), q.x + (int)(span[k] >> 16));
     } else {
-        for_rows(sm, nrec, vi, [&](int r, int ty, int a0, int a1) { put(s_depth[r], (uint32_t)r, ty, a0, a1); });
+        for_rows(sm, nrec, vi, 1u, [&](int r, int ty, int a0, int a1) { put(s_depth[r], (uint32_t)r, ty, a0, a1); });
     }
 }
 
