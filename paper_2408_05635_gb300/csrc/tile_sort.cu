@@ -17,9 +17,13 @@
 // Longer slices: a sample sort.  kSortKeys keys at equal strides are sorted as above, every
 // eighth is a splitter, the record ids are grouped by the intervals between them, and runs
 // of intervals that fit kSortKeys are sorted as above.  The splitters are whole keys, so
-// crowded or equal depths spread as evenly as others do; only if an interval still holds
-// more than kSortKeys, or beyond kSampleMax keys, does a bitonic network sort the slice in
-// global memory.
+// crowded or equal depths spread as evenly as others do.  An interval that holds more than
+// kSortKeys (from about 50k keys on a few, beyond 130k most) is put aside and split again by
+// samples of its own; only one that keeps more than seven eighths of its list, which takes equal
+// keys (stale ones, after a capacity overflow), goes through a bitonic network in global memory.  When one such interval,
+// or a list beyond 65,536 keys, sent the whole list through the network, a render of 60,000 in one
+// tile of 4,096 took 15.2 ms instead of 5.8, of 130,000 34.7 instead of 13.1 (the network inside
+// the compositor, with blocks of 256 threads: 9.7 and 22.1).
 //
 // Bound by latency and instruction issue (a list is read once: 15 MB for the window below).
 // As a kernel of its own it runs with many small blocks per SM, and leaves the compositors
@@ -39,7 +43,7 @@ constexpr int kFine = 1024;
 constexpr int kBucketMax = 128;            // comparing a fuller bucket's keys would cost more than the network
 constexpr int kCoarse = 128;               // intervals of a long list
 constexpr int kStride = kSortKeys / kCoarse;
-constexpr int kSampleMax = kCoarse * kSortKeys / 2;  // half a full buffer per interval on average
+constexpr int kTodo = 256;                 // intervals put aside: two levels of lists up to 2^27
 
 typedef unsigned long long Key;
 
@@ -86,6 +90,7 @@ struct SortSmem {
     Key split[kCoarse];
     uint32_t coarse[kCoarse];
     uint32_t lo[NT / 32], hi[NT / 32], sum[NT / 32], mx[NT / 32];
+    uint2 todo[kTodo];  // first place and number of keys of the intervals put aside
 };
 
 // Bucket of a depth: linear between the list's extremes.  Rounded subtraction and
@@ -214,10 +219,101 @@ __device__ __forceinline__ void intervals_of(const Key *split, const Key (&key)[
         for (int k = 0; k < PER; ++k) at[k] += split[at[k] + step - 1u] < key[k] ? step : 0u;
 }
 
+// More than kSortKeys keys.  A function of its own, so that its registers do not weigh on the short
+// lists (in the kernel's body: 80 bytes of spills a thread, and a render of 1M at 1200 x 680
+// 194.7 -> 198.3 us).
+template <int NT>
+__device__ __noinline__ void sort_long(const Rec *rec, uint32_t slots, Key *keys, uint32_t *out, int n, SortSmem<NT> &sm) {
+    const int tid = threadIdx.x;
+    Key key[kPer<NT>];
+    // the key of a record: its depth, as k_emit wrote it
+    const auto key_of = [&](uint32_t r) { return (Key)(r < slots ? __float_as_uint(rec[r].a.z) : 0u) << 32 | r; };
+    int waiting = 0;  // intervals put aside
+    uint32_t base = 0;
+    for (int m = n;;) {  // the m > kSortKeys keys from `base` on
+#pragma unroll
+        for (int k = 0; k < kPer<NT>; ++k)
+            key[k] = keys[base + (uint32_t)((uint64_t)(tid + k * NT) * (uint32_t)m / (uint32_t)kSortKeys)];
+        sort_keys(key, kSortKeys, sm, [&](uint32_t place, Key x) {
+            if (place % kStride == kStride - 1) sm.split[place / kStride] = x;
+        });
+        if (tid < kCoarse) sm.coarse[tid] = 0u;
+        __syncthreads();
+        bool crowded = false;  // an interval holds more than kSortKeys
+#pragma unroll 1
+        for (int pass = 0; pass < 2; ++pass) {  // count, then place
+            for (int i = tid; i < m; i += kSortKeys) {
+#pragma unroll
+                for (int k = 0; k < kPer<NT>; ++k)
+                    key[k] = keys[base + min(i + k * NT, m - 1)];
+                uint32_t at[kPer<NT>];
+                intervals_of(sm.split, key, at);
+#pragma unroll
+                for (int k = 0; k < kPer<NT>; ++k)
+                    if (i + k * NT < m) {
+                        const uint32_t slot = atomicAdd(&sm.coarse[at[k]], 1u);
+                        if (pass) out[base + slot] = (uint32_t)key[k];
+                    }
+            }
+            __syncthreads();
+            if (pass == 0) {
+                uint32_t mx = tid < kCoarse ? sm.coarse[tid] : 0u;
+                const uint32_t first = block_prefix(mx, mx, sm);
+                crowded = mx > (uint32_t)kSortKeys;
+                if (tid < kCoarse) sm.coarse[tid] = first;
+                __syncthreads();
+            }
+        }
+        if (crowded) {  // the keys in the intervals' order too, to be read by interval
+            for (int i = tid; i < m; i += NT) keys[base + i] = key_of(out[base + i]);
+            __syncthreads();
+        }
+        // coarse[k] is now the end of interval k: sort as many intervals at a time as fit
+        uint32_t done = 0;
+        for (int k = 0; done < (uint32_t)m;) {
+            const uint32_t size = sm.coarse[k] - done;
+            if (size > (uint32_t)kSortKeys) {
+                // (an eighth less at each level: the levels are few whatever the keys)
+                if (size > (uint32_t)(m - m / 8) || waiting == kTodo) {
+                    bitonic_sort<NT>(keys + base + done, (int)size);
+                    for (uint32_t i = tid; i < size; i += NT) out[base + done + i] = (uint32_t)keys[base + done + i];
+                } else {
+                    if (tid == 0) sm.todo[waiting] = make_uint2(base + done, size);
+                    ++waiting;
+                }
+                done += size;
+                ++k;
+                continue;
+            }
+            int l = k, e = kCoarse;  // the first interval that ends beyond the buffer (above k)
+            while (l < e) {
+                const int mid = (l + e) >> 1;
+                if (sm.coarse[mid] <= done + (uint32_t)kSortKeys) l = mid + 1; else e = mid;
+            }
+            const int c = (int)(sm.coarse[l - 1] - done);
+            uint32_t *to = out + base + done;
+#pragma unroll
+            for (int j = 0; j < kPer<NT>; ++j)
+                if (tid + j * NT < c) key[j] = key_of(to[tid + j * NT]);
+            sort_keys(key, c, sm, [&](uint32_t place, Key x) { to[place] = (uint32_t)x; });
+            done += (uint32_t)c;
+            k = l;
+        }
+        if (waiting == 0) return;
+        __syncthreads();  // (the list of intervals is written, and coarse read)
+        const uint2 next = sm.todo[--waiting];
+        base = next.x;
+        m = (int)next.y;
+    }
+}
+
 // Pair capacity per tile from which lists are taken to be long.  Blocks of 128 threads keep
 // more lists in flight (lists of 290 keys: 60 us against 80 with 256 threads; of 385: 40
 // against 53), blocks of 256 sort a long list sooner (513 keys on average, up to 1,858: 27
-// against 34 us; 1,847, up to 7,306: 88 against 113; 512 threads: 44 and 87).
+// against 34 us; 1,847, up to 7,306: 88 against 113; 512 threads: 44 and 87).  The capacity
+// stands for the keys, which only the device knows when the kernel is launched: with 1.25 pairs
+// reserved for one the line is at 513 keys a tile, with 1.05 at 610, and lists between those then
+// take the 34 us.
 constexpr uint32_t kLongLists = 640;
 
 // One block per tile, the longest lists first.  The key slice is left as it is or permuted, so the sort can be run
@@ -243,67 +339,7 @@ __global__ void __launch_bounds__(NT, 1280 / NT) k_sort_tiles(WsPtrs ws, Dims d)
         sort_keys(key, n, sm, [&](uint32_t place, Key x) { out[place] = (uint32_t)x; });
         return;
     }
-    bool network = n > kSampleMax;
-    if (!network) {
-#pragma unroll
-        for (int k = 0; k < kPer<NT>; ++k)
-            key[k] = keys[(uint32_t)(tid + k * NT) * (uint32_t)n / (uint32_t)kSortKeys];
-        sort_keys(key, kSortKeys, sm, [&](uint32_t place, Key x) {
-            if (place % kStride == kStride - 1) sm.split[place / kStride] = x;
-        });
-        if (tid < kCoarse) sm.coarse[tid] = 0u;
-        __syncthreads();
-        uint32_t run = 0;
-#pragma unroll 1
-        for (int pass = 0; pass < 2 && !network; ++pass) {  // count, then place
-            for (int i = tid; i < n; i += kSortKeys) {
-#pragma unroll
-                for (int k = 0; k < kPer<NT>; ++k)
-                    key[k] = keys[min(i + k * NT, n - 1)];
-                uint32_t at[kPer<NT>];
-                intervals_of(sm.split, key, at);
-#pragma unroll
-                for (int k = 0; k < kPer<NT>; ++k)
-                    if (i + k * NT < n) {
-                        const uint32_t slot = atomicAdd(&sm.coarse[at[k]], 1u);
-                        if (pass) out[slot] = (uint32_t)key[k];
-                    }
-            }
-            __syncthreads();
-            if (pass == 0) {
-                uint32_t mx = tid < kCoarse ? sm.coarse[tid] : 0u;
-                run = block_prefix(mx, mx, sm);
-                network = mx > (uint32_t)kSortKeys;
-                if (tid < kCoarse) sm.coarse[tid] = run;
-                __syncthreads();
-            }
-        }
-    }
-    if (network) {
-        bitonic_sort<NT>(keys, n);
-        for (int i = tid; i < n; i += NT) out[i] = (uint32_t)keys[i];
-        return;
-    }
-    // coarse[k] is now the end of interval k: sort as many intervals at a time as fit
-    uint32_t done = 0;
-    for (int k = 0; done < (uint32_t)n;) {
-        int l = k, e = kCoarse;  // the first interval that ends beyond the buffer (above k: none exceeds it)
-        while (l < e) {
-            const int mid = (l + e) >> 1;
-            if (sm.coarse[mid] <= done + (uint32_t)kSortKeys) l = mid + 1; else e = mid;
-        }
-        const int m = (int)(sm.coarse[l - 1] - done);
-        uint32_t *to = out + done;
-#pragma unroll
-        for (int j = 0; j < kPer<NT>; ++j)
-            if (tid + j * NT < m) {
-                const uint32_t r = to[tid + j * NT];  // the depth of its key is its record's
-                key[j] = (Key)(r < rec_slots(d) ? __float_as_uint(ws.rec[r].a.z) : 0u) << 32 | r;
-            }
-        sort_keys(key, m, sm, [&](uint32_t place, Key x) { to[place] = (uint32_t)x; });
-        done += (uint32_t)m;
-        k = l;
-    }
+    sort_long<NT>(ws.rec, rec_slots(d), keys, out, n, sm);
 }
 
 cudaError_t launch_sort_tiles(const WsPtrs &ws, const Dims &d, cudaStream_t st) {
