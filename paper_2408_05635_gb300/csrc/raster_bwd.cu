@@ -146,7 +146,9 @@ __global__ void __launch_bounds__(kTilePix, 4) k_backward(BackwardLaunch L) {
         const int nl = list_from_words(hits, sList[warp], wcnt, lane);
         // entries at byte offsets below lim are in front of this pixel's last contributor
         const int lim = (int)max(min((int64_t)last - b0, (int64_t)NB), (int64_t)0) * 16;
-        if (odd_planes(up)) {  // (asked again for every batch: the answer kept in a register cost spills)
+        // (asked again for every batch: the answer kept in a register cost spills.  A pose gradient is
+        // the sum over all Gaussians: not finite either way)
+        if (!POSE && odd_planes(up)) {
             const WalkState w = bwd_walk_odd<POSE>(sList[warp], nl, lim, sP0, sP1, sC, uv, pu_lo, pv_lo, thr, S.alpha_max, up,
                                                    WalkState{T, GB, n_eval, n_contrib}, buf, sAcc, lane);
             T = w.T;
