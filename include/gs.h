@@ -266,7 +266,7 @@ gs_status gs_sync_status(gs_ctx *ctx, void *stream, gs_counts *counts);
 /* Per-kernel device time of the last enqueued work, for profiling. */
 typedef struct {
     char name[24]; /* kernel (k_project, k_scan_tiles, k_emit, k_forward, k_backward,
-                      k_bproject, k_finalize) */
+                      k_bproject, k_finalize, k_track_tile, k_radix_sort, k_sort_tiles) */
     float ms;      /* CUDA-event time from the marker before this kernel's launch (which is the
                       end marker of the previous kernel when that one is also marked) to the
                       marker after it */
@@ -278,10 +278,10 @@ typedef struct {
 gs_status gs_set_profiling(gs_ctx *ctx, int32_t enable);
 
 /* Select the kernels bracketed by profiling markers: bit k of mask selects, in order,
- * k_project, k_scan_tiles, k_emit, k_forward, k_backward, k_bproject, k_finalize (0x7F:
- * all, as gs_set_profiling(ctx, 1); 0: off).  Unselected kernels get no events, so timing
- * one kernel disturbs the launch chain of the others less.  Errors: INVALID_ARG (a bit
- * above 6). */
+ * k_project, k_scan_tiles, k_emit, k_forward, k_backward, k_bproject, k_finalize,
+ * k_track_tile, k_radix_sort, k_sort_tiles (0x3FF: all, as gs_set_profiling(ctx, 1); 0:
+ * off).  Unselected kernels get no events, so timing one kernel disturbs the launch chain
+ * of the others less.  Errors: INVALID_ARG (a bit above 9). */
 gs_status gs_set_profiling_mask(gs_ctx *ctx, uint32_t mask);
 
 /* Synchronise on the last marker and return the per-kernel times of the work enqueued

@@ -130,7 +130,8 @@ gs_status cuda_fail(gs_ctx *ctx, cudaError_t e, const char *where) {
 }
 
 const char *const kKernelNames[] = {"k_project", "k_scan_tiles", "k_emit", "k_forward",
-                                    "k_backward", "k_bproject", "k_finalize", "k_track_tile", "k_radix_sort"};
+                                    "k_backward", "k_bproject", "k_finalize", "k_track_tile", "k_radix_sort",
+                                    "k_sort_tiles"};
 constexpr uint32_t kAllKernels = (1u << (sizeof(kKernelNames) / sizeof(kKernelNames[0]))) - 1u;
 
 bool selected(const gs_ctx *ctx, const char *name) {
@@ -403,6 +404,16 @@ cudaError_t enqueue_project(gs_ctx *ctx, const Problem &pr, const WsPtrs &w, con
     return mark(ctx, st, "k_radix_sort");
 }
 
+// Every tile's list in depth order, unless the device-wide radix sort (GS_SCHED_RADIX) has
+// already made it.
+cudaError_t enqueue_depth_order(gs_ctx *ctx, const Problem &pr, const WsPtrs &w, cudaStream_t st) {
+    if (pr.d.T == 0 || (pr.d.flags & GS_SCHED_RADIX)) return cudaSuccess;
+    cudaError_t e;
+    if ((e = mark_begin(ctx, st, "k_sort_tiles")) != cudaSuccess) return e;
+    if ((e = launch_sort_tiles(w, pr.d, st)) != cudaSuccess) return e;
+    return mark(ctx, st, "k_sort_tiles");
+}
+
 cudaError_t enqueue_forward(gs_ctx *ctx, const Problem &pr, const WsPtrs &w, const gs_targets *t, float *rgb,
                             float *depth, float *sil, cudaStream_t st) {
     cudaError_t e;
@@ -416,6 +427,7 @@ cudaError_t enqueue_forward(gs_ctx *ctx, const Problem &pr, const WsPtrs &w, con
     F.t_rgb = t ? t->rgb : nullptr;
     F.t_depth = t ? t->depth : nullptr;
     F.t_prior = t ? t->depth_prior : nullptr;
+    if ((e = enqueue_depth_order(ctx, pr, w, st)) != cudaSuccess) return e;
     if ((e = mark_begin(ctx, st, "k_forward")) != cudaSuccess) return e;
     if ((e = launch_forward(F, st)) != cudaSuccess) return e;
     return mark(ctx, st, "k_forward");
@@ -434,6 +446,7 @@ cudaError_t enqueue_compositing(gs_ctx *ctx, const Problem &pr, const WsPtrs &w,
         K.t_rgb = t->rgb;
         K.t_depth = t->depth;
         K.t_prior = t->depth_prior;
+        if ((r = enqueue_depth_order(ctx, pr, w, st)) != cudaSuccess) return r;
         if ((r = mark_begin(ctx, st, "k_track_tile")) != cudaSuccess) return r;
         if ((r = launch_track_tile(K, st)) != cudaSuccess) return r;
         return mark(ctx, st, "k_track_tile");

@@ -631,11 +631,6 @@ cudaError_t launch_project(const ProjectLaunch &L, cudaStream_t st);
 cudaError_t launch_scan_tiles(const WsPtrs &ws, const Dims &d, cudaStream_t st);
 cudaError_t launch_emit(const WsPtrs &ws, const Dims &d, cudaStream_t st);
 cudaError_t launch_sort_tiles(const WsPtrs &ws, const Dims &d, cudaStream_t st);
-// Before a forward: every tile's list in depth order, unless the device-wide radix sort
-// (GS_SCHED_RADIX) has already made it.
-inline cudaError_t launch_depth_order(const WsPtrs &ws, const Dims &d, cudaStream_t st) {
-    return d.flags & GS_SCHED_RADIX ? cudaSuccess : launch_sort_tiles(ws, d, st);
-}
 
 struct ForwardLaunch {
     WsPtrs ws;

@@ -170,6 +170,7 @@ extern "C" gs_status gs_render_static(const gs_config *cfg, const gs_gaussians *
     F.t_rgb = targets ? targets->rgb : nullptr;
     F.t_depth = targets ? targets->depth : nullptr;
     F.t_prior = targets ? targets->depth_prior : nullptr;
+    if (launch_sort_tiles(w, d, st) != cudaSuccess) return GS_ERR_CUDA;
     if (launch_forward(F, st) != cudaSuccess) return GS_ERR_CUDA;
     if (loss) {
         FinalizeLaunch Z{};

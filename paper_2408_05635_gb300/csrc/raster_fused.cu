@@ -267,8 +267,7 @@ cudaError_t launch_track_tile(const TrackTileLaunch &L, cudaStream_t st) {
     const uint32_t nb = L.d.fwd_batch ? L.d.fwd_batch : (uint32_t)kBatch;
     if (nb > tile_threads(L.d) || (L.d.bwd_batch ? L.d.bwd_batch : (uint32_t)kBatch) != nb)
         return cudaErrorInvalidValue;
-    cudaError_t e = launch_depth_order(L.ws, L.d, st);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     switch (nb) {
         case 256: e = launch_track_tile_lw<256>(L, st); break;
         case 128: e = launch_track_tile_lw<128>(L, st); break;

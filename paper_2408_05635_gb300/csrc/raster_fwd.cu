@@ -204,8 +204,7 @@ cudaError_t launch_forward(const ForwardLaunch &L, cudaStream_t st) {
     // a batch stages at most one Gaussian per thread of the tile block
     const uint32_t nb = L.d.fwd_batch ? L.d.fwd_batch : (uint32_t)kBatch;
     if (nb > tile_threads(L.d)) return cudaErrorInvalidValue;
-    cudaError_t e = launch_depth_order(L.ws, L.d, st);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     switch (L.d.fwd_batch) {
         case 0:
         case 256: e = launch_forward_lw<256>(L, st); break;

@@ -297,7 +297,7 @@ def gs_set_profiling(ctx, enable: bool) -> None:
 
 
 KERNELS = ("k_project", "k_scan_tiles", "k_emit", "k_forward", "k_backward", "k_bproject", "k_finalize",
-           "k_track_tile", "k_radix_sort")
+           "k_track_tile", "k_radix_sort", "k_sort_tiles")
 
 
 def gs_set_profiling_mask(ctx, kernels) -> None:
