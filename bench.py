@@ -10,7 +10,9 @@ launched from the library's CUDA graph).
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 
-Rank 0 prints one JSON line.  With N > 1 (torchrun) every rank tracks its own frame:
+Rank 0 prints one JSON line with the headline figures on standard output, and before it the whole
+record (every leg, its tuning tables, the accuracy against the oracle) as one JSON line on
+standard error.  With N > 1 (torchrun) every rank tracks its own frame:
 replicas only, weak scaling.  ``--impl reference`` times the FP64 CPU oracle on the
 same workload (bounded samples per step) on the host cores.
 """
@@ -822,6 +824,41 @@ def run_reference(a, rank, world):
     print(json.dumps(line), flush=True)
 
 
+def headline(record: dict) -> dict:
+    """The figures of the record that fit a line a log's tail keeps whole (under 2,500
+    characters): the timed workload in full, one figure or two of every other leg."""
+    def cut(d, *keys):
+        return {k: d[k] for k in keys if k in d}
+
+    out = cut(record, "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "tracking_iters_per_s", "gpu_launches", "clocks", "kernels_us", "pairs_per_step")
+    out["config"] = cut(record["config"], "workload", "gaussians", "pairs", "records", "l2", "parallelism")
+    out["config"]["schedule"] = (record["config"].get("launch_schedule") or {}).get("schedule")
+    out["e2e"] = cut(record["e2e"], "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")
+    out["e2e"]["copied_upload"] = record["e2e"]["copied_upload"]["value"]
+    if record.get("roofline"):
+        out["roofline"] = cut(record["roofline"], "kernel", "bound", "achieved", "peak", "unit", "frac", "traffic")
+    legs = {}
+    if "isotropic" in record:
+        legs["isotropic_us_per_iter"] = record["isotropic"]["isotropic"]["us_per_iter"]
+    if "batched" in record:
+        legs["batched_512_views_mpix_per_s"] = round(record["batched"]["batched_bf16"]["mpix_per_s"], 1)
+        legs["batched_speedup_vs_tuned_plain"] = round(record["batched"]["speedup_vs_tuned_plain"], 3)
+    if "mapping" in record:
+        legs["mapping_window_ms"] = min(c["ms_per_window"] for c in record["mapping"]["chunks"].values())
+    for k, v in record.get("sequence", {}).items():
+        if isinstance(v, dict):
+            legs[f"{k}_ms_per_frame"] = v["ms_per_frame"]
+    if legs:
+        out["legs"] = legs
+    if "cpu_baseline" in record:
+        out["cpu_baseline"] = cut(record["cpu_baseline"], "value", "unit", "cores", "kind", "sample")
+        frame = record["cpu_baseline"].get("accuracy_vs_oracle", {}).get("tracking_frame")
+        if frame:
+            out["accuracy_vs_oracle"] = cut(frame, "max_err_unflagged", "loss_rel_err", "pose_grad_rel_err")
+    return out
+
+
 def sm_count() -> int:
     """Streaming multiprocessors of the current GPU, read from the device."""
     import torch
@@ -845,8 +882,9 @@ def kernel_rooflines(kern_ms: dict, n_gauss: int, views: int, attr_bytes: int, r
     algorithmic bytes or FLOPs per launch (from the work counted on the device) over its
     CUDA-event time (markers around every kernel, so each time includes its launch gap),
     as a fraction of the measured HBM copy bandwidth or of the FP32 FMA peak at the
-    sampled SM clock.  k_scan_tiles (one block) and k_finalize (a chain of dependent
-    steps) are latency-bound: their times are reported without a roofline."""
+    sampled SM clock.  k_scan_tiles (one block), k_sort_tiles (a few dependent phases a block)
+    and k_finalize (a chain of dependent steps) are latency-bound: their times are reported
+    without a roofline."""
     hbm, hbm_from = hbm_peak_gbs()
     n_sm = n_sm or sm_count()
     fp32 = n_sm * FP32_LANES * 2 * mhz * 1e6 / 1e12
@@ -1105,7 +1143,8 @@ def main():
             t0 = time.perf_counter()
             line["cpu_baseline"]["accuracy_vs_oracle"] = accuracy_vs_oracle(dev, stream)
             line["cpu_baseline"]["accuracy_vs_oracle"]["seconds"] = round(time.perf_counter() - t0, 1)
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     if world > 1:
         dist.destroy_process_group()
 
