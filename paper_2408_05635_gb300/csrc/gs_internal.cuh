@@ -33,8 +33,8 @@ constexpr int kCell = kBlock;             // Gaussians (and record slots) per ce
 constexpr int kBatch = 256;               // default (and largest) compositing batch depth
 // The compositors are compiled for batch depths 64, 128 and 256 (Gaussians staged into
 // shared memory per batch).  The first NB threads of the tile block stage one Gaussian
-// each and own one accumulator row each, and the per-warp lists hold batch positions as
-// bytes: NB must not exceed 256 nor the tile's thread count (the host checks the latter).
+// each and own one accumulator row each, and the per-warp lists hold 16 times a batch position
+// in 16 bits: NB must not exceed 256 nor the tile's thread count (the host checks the latter).
 static_assert(kBatch <= kTilePix && kBatch <= 256, "a batch stages at most one Gaussian per tile thread");
 constexpr int kSubMax = 4;                // most per-tile sub-buckets a workspace is laid out for
 

@@ -3,10 +3,11 @@
 //
 // Three launches.  k_pyramid makes the four coarser scales by 2 x 2 average pooling.
 // k_ssim_terms takes the local statistics of every scale and channel at once: a window
-// position's moments under the 11 x 11 Gaussian window (sigma 1.5), centred on the window's
-// middle pixel so that the variances do not cancel in FP32 -- which rules out separable
-// passes, since every position has its own centre -- are 121 taps of nine FP32 operations,
-// and that arithmetic bounds the kernel.  A thread takes two positions eight rows apart in
+// position's moments under the 11 x 11 Gaussian window (sigma 1.5) are centred on the window's
+// middle pixel so that the variances do not cancel in FP32.  Every position has its own centre,
+// so they are taken position by position: 121 taps of nine FP32 operations, and that
+// arithmetic bounds the kernel.  (Row moments about a pixel of the row, shifted to the
+// window's middle while the rows are added, would be separable; not built.)  A thread takes two positions eight rows apart in
 // the two lanes of FP32 pair instructions, from a shared tile that stores the two rows
 // interleaved.  The term itself, (2 cov + C2) / (var + var + C2), and its sum are double-float
 // on the FP32 pipes (about 46 bits): in FP64 they took longer than the window.

@@ -4,7 +4,7 @@
 // Eqs. 2-4.
 //
 // It computes what k_forward<loss> followed by k_backward<pose-only> compute (the same
-// footprint code, the same per-warp lists, the same reduce-scatter; see raster_fwd.cu and
+// footprint code, the same per-warp lists, the same transposed sums; see raster_fwd.cu and
 // raster_bwd.cu for the arithmetic), with three differences in how the work is laid out:
 //   - each pixel's upstream gradient, final transmittance and last contributor stay in
 //     registers between the walks and are not written to the workspace (the pass consumes
