@@ -16,7 +16,8 @@
 // one block, a thread adding hundreds of terms, up to 14 off; here 1.9 (six images of noise).
 // Errors outside (2^-40, 2^40) take the FP64 path: inside, the squares of eight threads' pixels
 // add to less than FP32's 2^128 for up to 2^43 pixels a thread, and a square's rounding error is a
-// normal number.  Measured at 640 x 480 (9.8 MB through 16 SMs): 26 us (21 with two floats).
+// normal number.  Measured at 640 x 480 (9.8 MB through 16 SMs): 26 us (21 with two floats), bound by
+// instruction issue (68 % of the 16 SMs' cycles) and the loads.
 #include <cooperative_groups.h>
 
 #include "gs_internal.cuh"
@@ -36,8 +37,8 @@ __device__ __forceinline__ float two_sum(float a, float b, float &e) {
     return s;
 }
 
-// The same for a, b >= 0: Dekker's Fast2Sum on the ordered pair (the comparisons run beside the
-// FP32 pipe, which bounds the pass).
+// The same for a, b >= 0: Dekker's Fast2Sum on the ordered pair (five instructions for six, two of
+// them beside the FP32 pipe).
 __device__ __forceinline__ float two_sum_pos(float a, float b, float &e) {
     const float x = fmaxf(a, b), y = fminf(a, b);
     const float s = __fadd_rn(x, y);
