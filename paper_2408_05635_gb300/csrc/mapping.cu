@@ -115,8 +115,9 @@ __device__ uint32_t block_rank(bool flag, uint32_t &count) {
 // results are those of FP64 rounded to FP32: a pair known to within `err` decides the rounding
 // unless the point halfway between two FP32 values lies inside that (nearest), and then, or
 // where the pairs leave FP32's range, the pixel is unprojected in FP64.
-// Measured in the same call: 60.4 us for the 307,200 pixels of a 640 x 480 frame (pairs with no such
-// check 60.1, all in FP64 94.6), 93 for 1200 x 680 (87, 199); about one pixel in 2,000 goes to FP64.
+// Measured in the same call: 57.5 us for the 307,200 pixels of a 640 x 480 frame (pairs with no such
+// check 56.2, all in FP64 94.6), 87.7 for 1200 x 680 (85.3, 199); about one pixel in 3,000 has a value that goes
+// to FP64.
 using gsk::DF;
 using gsk::df_add;
 
@@ -176,6 +177,7 @@ struct AddLaunch {
     float sil_add;
     double fx, fy, cx, cy;
     DF ifx, ify, ncx, ncy, inv_f;  // 1 / fx, 1 / fy, -cx, -cy, 2 / (fx + fy)
+    double ifx64, ify64, inv_f64;
     bool pairs;                    // the camera lies inside the pairs' range
     int32_t width, height;
     uint32_t *counts;  // scratch: one word per block
@@ -223,6 +225,15 @@ __device__ __noinline__ void unproject_fp64(const AddLaunch &L, const double *R,
     ls = (float)log(d / (0.5 * (L.fx + L.fy)));
 }
 
+// The means alone, of a pixel inside the pairs' range: with the reciprocals of the focal lengths,
+// since FP64 divisions would make a block wait for 3 us.
+__device__ __noinline__ void unproject_near_tie(const AddLaunch &L, const double *Rt, int u, int v, double d, float (&mean)[3]) {
+    const double xc0 = ((double)u - L.cx) * L.ifx64 * d - Rt[9];
+    const double xc1 = ((double)v - L.cy) * L.ify64 * d - Rt[10];
+    const double xc2 = d - Rt[11];
+    for (int k = 0; k < 3; ++k) mean[k] = (float)(Rt[k] * xc0 + Rt[3 + k] * xc1 + Rt[6 + k] * xc2);
+}
+
 // `values` consecutive values of one output array, value(i) the i-th; consecutive threads
 // take consecutive values.
 template <class T, class F>
@@ -251,26 +262,29 @@ __global__ void __launch_bounds__(kCompactThreads, 2) k_add_emit(AddLaunch L) {
         const int v = (int)(p / L.width), u = (int)(p - (int64_t)v * L.width);
         const float d = L.depth[p];
         float mean[3], ls;
-        bool sure = L.pairs && d > 0x1p-60f && d < 0x1p60f;
-        if (sure) {
+        if (L.pairs && d > 0x1p-60f && d < 0x1p60f) {
+            bool sure = true;
             const DF D{d, 0.f};
             const DF x0 = df_add(df_mul(df_mul(df_add(DF{(float)u, 0.f}, L.ncx), L.ifx), D), s_nt[0]);
             const DF x1 = df_add(df_mul(df_mul(df_add(DF{(float)v, 0.f}, L.ncy), L.ify), D), s_nt[1]);
             const DF x2 = df_add(D, s_nt[2]);
-            // every term of a mean is at most `size`, and the operations on its way lose a few 2^-46
+            // every term of a mean is at most `size`; on its way are three products and four sums of
+            // pairs (2^-46 and 2^-46.5 of it each) and three rounded factors (2^-48): 2^-43.3 together
             const float size = ((float)u + fabsf(L.ncx.hi)) * L.ifx.hi * d + ((float)v + fabsf(L.ncy.hi)) * L.ify.hi * d + d +
                                fabsf(s_nt[0].hi) + fabsf(s_nt[1].hi) + fabsf(s_nt[2].hi);
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const DF x = df_add(df_add(df_mul(s_R[k], x0), df_mul(s_R[3 + k], x1)), df_mul(s_R[6 + k], x2));
                 mean[k] = x.hi;
-                sure = sure && nearest(x, 0x1p-42f * size);
+                sure = sure && nearest(x, 0x1p-43f * size);
             }
             const DF ln = log_pair(df_mul(D, L.inv_f));
             ls = ln.hi;
-            sure = sure && nearest(ln, 0x1p-40f * (fabsf(ls) + 0.5f));
+            if (!sure) unproject_near_tie(L, L.Rt, u, v, (double)d, mean);
+            if (!nearest(ln, 0x1p-40f * (fabsf(ls) + 0.5f))) ls = (float)log((double)d * L.inv_f64);
+        } else {
+            unproject_fp64(L, L.Rt, L.Rt + 9, u, v, (double)d, mean, ls);
         }
-        if (!sure) unproject_fp64(L, L.Rt, L.Rt + 9, u, v, (double)d, mean, ls);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             s_mean[3 * r + k] = mean[k];
@@ -542,6 +556,9 @@ gs_status gs_map_add(const gs_map_config *cfg, const gs_map *map, int64_t *n, co
     L.ncx = df_host(-cam->cx);
     L.ncy = df_host(-cam->cy);
     L.inv_f = df_host(2.0 / (cam->fx + cam->fy));
+    L.ifx64 = 1.0 / cam->fx;
+    L.ify64 = 1.0 / cam->fy;
+    L.inv_f64 = 2.0 / (cam->fx + cam->fy);
     // pixel coordinates exact in FP32, no underflow in a product's low part, no overflow of one
     const auto in_range = [](double x) { return x > 0x1p-30 && x < 0x1p30; };
     L.pairs = in_range(cam->fx) && in_range(cam->fy) && std::fabs(cam->cx) < 0x1p30 && std::fabs(cam->cy) < 0x1p30 &&
