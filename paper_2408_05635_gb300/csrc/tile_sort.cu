@@ -19,11 +19,12 @@
 // of intervals that fit kSortKeys are sorted as above.  The splitters are whole keys, so
 // crowded or equal depths spread as evenly as others do.  An interval that holds more than
 // kSortKeys (from about 50k keys on a few, beyond 130k most) is put aside and split again by
-// samples of its own; only one that keeps more than seven eighths of its list, which takes equal
-// keys (stale ones, after a capacity overflow), goes through a bitonic network in global memory.  When one such interval,
-// or a list beyond 65,536 keys, sent the whole list through the network, a render of 60,000 in one
-// tile of 4,096 took 15.2 ms instead of 5.8, of 130,000 34.7 instead of 13.1 (the network inside
-// the compositor, with blocks of 256 threads: 9.7 and 22.1).
+// samples of its own.  Only where an interval keeps more than seven eighths of its range, which
+// takes equal keys (stale ones, after a capacity overflow), does a bitonic network in global
+// memory sort the range.  When one long interval, or a list beyond 65,536 keys, sent the whole
+// list through the network, a render of 60,000 in one tile of 4,096 took 15.2 ms instead of 5.8,
+// of 130,000 34.7 instead of 13.2 (the network inside the compositor, with blocks of 256
+// threads: 9.7 and 22.1).
 //
 // Bound by latency and instruction issue (a list is read once: 15 MB for the window below).
 // As a kernel of its own it runs with many small blocks per SM, and leaves the compositors
@@ -43,7 +44,7 @@ constexpr int kFine = 1024;
 constexpr int kBucketMax = 128;            // comparing a fuller bucket's keys would cost more than the network
 constexpr int kCoarse = 128;               // intervals of a long list
 constexpr int kStride = kSortKeys / kCoarse;
-constexpr int kTodo = 256;                 // intervals put aside: two levels of lists up to 2^27
+constexpr int kTodo = 256;                 // intervals put aside: those of two levels
 
 typedef unsigned long long Key;
 
@@ -92,6 +93,14 @@ struct SortSmem {
     uint32_t lo[NT / 32], hi[NT / 32], sum[NT / 32], mx[NT / 32];
     uint2 todo[kTodo];  // first place and number of keys of the intervals put aside
 };
+
+// The block's shared memory, by name in every function that uses it (through a reference it would be
+// addressed as any memory).
+template <int NT>
+__device__ __forceinline__ SortSmem<NT> &sort_smem() {
+    __shared__ SortSmem<NT> sm;
+    return sm;
+}
 
 // Bucket of a depth: linear between the list's extremes.  Rounded subtraction and
 // multiplication are monotone, so a smaller depth never lands in a later bucket (equal
@@ -219,91 +228,108 @@ __device__ __forceinline__ void intervals_of(const Key *split, const Key (&key)[
         for (int k = 0; k < PER; ++k) at[k] += split[at[k] + step - 1u] < key[k] ? step : 0u;
 }
 
-// More than kSortKeys keys.  A function of its own, so that its registers do not weigh on the short
-// lists (in the kernel's body: 80 bytes of spills a thread, and a render of 1M at 1200 x 680
-// 194.7 -> 198.3 us).
+// The key of a record: its depth, as k_emit wrote it.
+__device__ __forceinline__ Key key_of(const Rec *rec, uint32_t slots, uint32_t r) {
+    return (Key)(r < slots ? __float_as_uint(rec[r].a.z) : 0u) << 32 | r;
+}
+
+// The m > kSortKeys keys of a list's slice from place `base` on: their record ids grouped by sampled
+// intervals and sorted in those that fit; the others are put aside after the `waiting` ones there.
+// Returns how many wait (more than kTodo: the last ones are not noted).
 template <int NT>
-__device__ __noinline__ void sort_long(const Rec *rec, uint32_t slots, Key *keys, uint32_t *out, int n, SortSmem<NT> &sm) {
+__device__ __forceinline__ int sort_level(const Rec *rec, uint32_t slots, const Key *keys, uint32_t *out, int m, uint32_t base,
+                                          int waiting, SortSmem<NT> &sm) {
     const int tid = threadIdx.x;
     Key key[kPer<NT>];
-    // the key of a record: its depth, as k_emit wrote it
-    const auto key_of = [&](uint32_t r) { return (Key)(r < slots ? __float_as_uint(rec[r].a.z) : 0u) << 32 | r; };
-    int waiting = 0;  // intervals put aside
-    uint32_t base = 0;
-    for (int m = n;;) {  // the m > kSortKeys keys from `base` on
 #pragma unroll
-        for (int k = 0; k < kPer<NT>; ++k)
-            key[k] = keys[base + (uint32_t)((uint64_t)(tid + k * NT) * (uint32_t)m / (uint32_t)kSortKeys)];
-        sort_keys(key, kSortKeys, sm, [&](uint32_t place, Key x) {
-            if (place % kStride == kStride - 1) sm.split[place / kStride] = x;
-        });
-        if (tid < kCoarse) sm.coarse[tid] = 0u;
-        __syncthreads();
-        bool crowded = false;  // an interval holds more than kSortKeys
+    for (int k = 0; k < kPer<NT>; ++k)
+        key[k] = keys[(uint32_t)((uint64_t)(tid + k * NT) * (uint32_t)m / (uint32_t)kSortKeys)];
+    sort_keys(key, kSortKeys, sm, [&](uint32_t place, Key x) {
+        if (place % kStride == kStride - 1) sm.split[place / kStride] = x;
+    });
+    if (tid < kCoarse) sm.coarse[tid] = 0u;
+    __syncthreads();
 #pragma unroll 1
-        for (int pass = 0; pass < 2; ++pass) {  // count, then place
-            for (int i = tid; i < m; i += kSortKeys) {
+    for (int pass = 0; pass < 2; ++pass) {  // count, then place
+        for (int i = tid; i < m; i += kSortKeys) {
 #pragma unroll
-                for (int k = 0; k < kPer<NT>; ++k)
-                    key[k] = keys[base + min(i + k * NT, m - 1)];
-                uint32_t at[kPer<NT>];
-                intervals_of(sm.split, key, at);
+            for (int k = 0; k < kPer<NT>; ++k)
+                key[k] = keys[min(i + k * NT, m - 1)];
+            uint32_t at[kPer<NT>];
+            intervals_of(sm.split, key, at);
 #pragma unroll
-                for (int k = 0; k < kPer<NT>; ++k)
-                    if (i + k * NT < m) {
-                        const uint32_t slot = atomicAdd(&sm.coarse[at[k]], 1u);
-                        if (pass) out[base + slot] = (uint32_t)key[k];
-                    }
-            }
-            __syncthreads();
-            if (pass == 0) {
-                uint32_t mx = tid < kCoarse ? sm.coarse[tid] : 0u;
-                const uint32_t first = block_prefix(mx, mx, sm);
-                crowded = mx > (uint32_t)kSortKeys;
-                if (tid < kCoarse) sm.coarse[tid] = first;
-                __syncthreads();
-            }
-        }
-        if (crowded) {  // the keys in the intervals' order too, to be read by interval
-            for (int i = tid; i < m; i += NT) keys[base + i] = key_of(out[base + i]);
-            __syncthreads();
-        }
-        // coarse[k] is now the end of interval k: sort as many intervals at a time as fit
-        uint32_t done = 0;
-        for (int k = 0; done < (uint32_t)m;) {
-            const uint32_t size = sm.coarse[k] - done;
-            if (size > (uint32_t)kSortKeys) {
-                // (an eighth less at each level: the levels are few whatever the keys)
-                if (size > (uint32_t)(m - m / 8) || waiting == kTodo) {
-                    bitonic_sort<NT>(keys + base + done, (int)size);
-                    for (uint32_t i = tid; i < size; i += NT) out[base + done + i] = (uint32_t)keys[base + done + i];
-                } else {
-                    if (tid == 0) sm.todo[waiting] = make_uint2(base + done, size);
-                    ++waiting;
+            for (int k = 0; k < kPer<NT>; ++k)
+                if (i + k * NT < m) {
+                    const uint32_t slot = atomicAdd(&sm.coarse[at[k]], 1u);
+                    if (pass) out[slot] = (uint32_t)key[k];
                 }
-                done += size;
-                ++k;
-                continue;
-            }
-            int l = k, e = kCoarse;  // the first interval that ends beyond the buffer (above k)
-            while (l < e) {
-                const int mid = (l + e) >> 1;
-                if (sm.coarse[mid] <= done + (uint32_t)kSortKeys) l = mid + 1; else e = mid;
-            }
-            const int c = (int)(sm.coarse[l - 1] - done);
-            uint32_t *to = out + base + done;
+        }
+        __syncthreads();
+        if (pass == 0) {
+            uint32_t mx = tid < kCoarse ? sm.coarse[tid] : 0u;
+            const uint32_t first = block_prefix(mx, mx, sm);
+            if (tid < kCoarse) sm.coarse[tid] = first;
+            __syncthreads();
+        }
+    }
+    // coarse[k] is now the end of interval k: sort as many intervals at a time as fit
+    uint32_t done = 0;
+    for (int k = 0; done < (uint32_t)m;) {
+        int l = k, e = kCoarse;  // the first interval that ends beyond the buffer
+        while (l < e) {
+            const int mid = (l + e) >> 1;
+            if (sm.coarse[mid] <= done + (uint32_t)kSortKeys) l = mid + 1; else e = mid;
+        }
+        if (l == k) {  // interval k alone is too long
+            const uint32_t size = sm.coarse[k] - done;
+            if (tid == 0 && waiting < kTodo) sm.todo[waiting] = make_uint2(base + done, size);
+            ++waiting;
+            done += size;
+            ++k;
+            continue;
+        }
+        const int c = (int)(sm.coarse[l - 1] - done);
+        uint32_t *to = out + done;
 #pragma unroll
-            for (int j = 0; j < kPer<NT>; ++j)
-                if (tid + j * NT < c) key[j] = key_of(to[tid + j * NT]);
-            sort_keys(key, c, sm, [&](uint32_t place, Key x) { to[place] = (uint32_t)x; });
-            done += (uint32_t)c;
-            k = l;
+        for (int j = 0; j < kPer<NT>; ++j)
+            if (tid + j * NT < c) key[j] = key_of(rec, slots, to[tid + j * NT]);
+        sort_keys(key, c, sm, [&](uint32_t place, Key x) { to[place] = (uint32_t)x; });
+        done += (uint32_t)c;
+        k = l;
+    }
+    return waiting;
+}
+
+// The intervals that the first level over a list's n keys put aside, and theirs.  Each is split by
+// samples of its own once the keys stand in the intervals' order; where an interval keeps more
+// than seven eighths of its range (equal keys), the range goes through the network, so the levels are few
+// whatever the keys.  A function of its own: in the kernel's body it cost the lists that need none of it
+// (80 bytes of spills a thread; a render of 1M at 1200 x 680, longest list 1,224, 194.7 -> 198.3 us).
+template <int NT>
+__device__ __noinline__ void sort_waiting(const Rec *rec, uint32_t slots, Key *keys, uint32_t *out, int n, int waiting) {
+    SortSmem<NT> &sm = sort_smem<NT>();
+    uint32_t base = 0;
+    int m = n, before = 0;  // the range just split; [before, waiting): its intervals
+    for (;;) {
+        __syncthreads();  // (the intervals are noted, and coarse read)
+        if (waiting > before) {
+            bool split = waiting <= kTodo;
+            for (int w = before; split && w < waiting; ++w) split = sm.todo[w].y <= (uint32_t)(m - m / 8);
+            if (split) {
+                for (int i = threadIdx.x; i < m; i += NT) keys[base + i] = key_of(rec, slots, out[base + i]);
+            } else {
+                bitonic_sort<NT>(keys + base, m);
+                for (int i = threadIdx.x; i < m; i += NT) out[base + i] = (uint32_t)keys[base + i];
+                waiting = before;
+            }
+            __syncthreads();
         }
         if (waiting == 0) return;
-        __syncthreads();  // (the list of intervals is written, and coarse read)
         const uint2 next = sm.todo[--waiting];
         base = next.x;
         m = (int)next.y;
+        before = waiting;
+        waiting = sort_level<NT>(rec, slots, keys + base, out + base, m, base, waiting, sm);
     }
 }
 
@@ -324,7 +350,7 @@ __global__ void __launch_bounds__(NT, 1280 / NT) k_sort_tiles(WsPtrs ws, Dims d)
     // no early griddep_launch_dependents: the compositor's longest tiles, launched first,
     // would crowd onto the SMs that free first
     griddep_wait();  // the predecessor's results are visible from here on
-    __shared__ SortSmem<NT> sm;
+    SortSmem<NT> &sm = sort_smem<NT>();
     const int tid = threadIdx.x;
     uint32_t start;
     const int n = (int)tile_entries(ws, d, ws.tile_order[blockIdx.x], start);
@@ -339,7 +365,8 @@ __global__ void __launch_bounds__(NT, 1280 / NT) k_sort_tiles(WsPtrs ws, Dims d)
         sort_keys(key, n, sm, [&](uint32_t place, Key x) { out[place] = (uint32_t)x; });
         return;
     }
-    sort_long<NT>(ws.rec, rec_slots(d), keys, out, n, sm);
+    const int waiting = sort_level<NT>(ws.rec, rec_slots(d), keys, out, n, 0u, 0, sm);
+    if (waiting > 0) sort_waiting<NT>(ws.rec, rec_slots(d), keys, out, n, waiting);
 }
 
 cudaError_t launch_sort_tiles(const WsPtrs &ws, const Dims &d, cudaStream_t st) {
