@@ -11,7 +11,7 @@
 // (consecutive threads, consecutive words) instead of a row of three or four values per
 // thread: at 1M Gaussians with moments and an FP16 copy k_prune_emit takes 73 us against 108
 // (425 MB: 63 us at the copy rate), and for 154 k new Gaussians of a 640 x 480 frame
-// k_add_emit 19 us against 44 (part of that was FP64, below).  No block waits on another, and the live count stays on the device.
+// k_add_emit 20 us against 44 (part of that was FP64, below).  No block waits on another, and the live count stays on the device.
 #include <cuda_fp16.h>
 
 #include <algorithm>
